@@ -786,7 +786,7 @@ cc_status cc_load_labels(cc_ctx* c, const int32_t* labels) {
     if (e == cudaSuccess) e = cudaMemsetAsync(&c->ds->roots, 0, sizeof(unsigned long long), c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cc_load_labels");
     cc_status s = run(c, CC_K_LOAD, "load_labels(validate)", [&] {
-        return cc::launch_validate_labels(labels, c->n, c->ds, 256, c->stream);
+        return cc::launch_validate_labels(labels, c->n, c->ds, c->stream);
     });
     if (s != CC_OK) return s;
     cc::DevState h;
@@ -1280,7 +1280,7 @@ cc_status cc_load_forest(cc_ctx* c, const int32_t* parent) {
     CC_DEVICE(c);
     cudaError_t e = cudaMemsetAsync(&c->ds->labels_bad, 0, sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(&c->ds->roots, 0, sizeof(unsigned long long), c->stream);
-    if (e == cudaSuccess) e = cc::launch_validate_forest(parent, c->n, c->ds, 256, c->stream);
+    if (e == cudaSuccess) e = cc::launch_validate_forest(parent, c->n, c->ds, c->stream);
     cc::DevState h;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, c->ds, sizeof h, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -241,10 +241,9 @@ cudaError_t launch_filter_roots(const int* res, int64_t k, int* a2, unsigned* m2
                                 unsigned long long* best, int block, cudaStream_t s);
 
 // Checks 0 <= p[v] <= v (and no more); counts roots.
-cudaError_t launch_validate_forest(const int* p, int64_t n, DevState* ds, int block, cudaStream_t s);
+cudaError_t launch_validate_forest(const int* p, int64_t n, DevState* ds, cudaStream_t s);
 
 // Checks 0 <= lab[v] <= v and lab[lab[v]] == lab[v]; counts roots.
-cudaError_t launch_validate_labels(const int* lab, int64_t n, DevState* ds, int block,
-                                   cudaStream_t s);
+cudaError_t launch_validate_labels(const int* lab, int64_t n, DevState* ds, cudaStream_t s);
 
 }  // namespace cc

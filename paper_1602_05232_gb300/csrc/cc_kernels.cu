@@ -1205,42 +1205,69 @@ cudaError_t launch_compress_touched(int* parent, int n, const int* edges, int64_
 
 // ------------------------------------------------------- label validation
 
-__global__ void __launch_bounds__(1024)
-k_validate_labels(const int* __restrict__ lab, int64_t n, DevState* __restrict__ ds) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int root = 0;
-    if (v < n) {
-        const int l = lab[v];
-        const bool good = l >= 0 && (int64_t)l <= v && lab[l] == l;
-        if (!good) atomicOr(&ds->labels_bad, 1u);
-        root = good && (int64_t)l == v;
+// Checks an array loaded from outside and counts its roots: LABELS wants
+// 0 <= a[v] <= v and a[a[v]] == a[v], else only 0 <= a[v] <= v. Bound by the
+// stream of n ids plus, for labels, the gather of each label's own label
+// (skipped at a root; one hot line where a giant component holds most ids).
+// Four ids per thread and step (one 16-byte load where the array allows it),
+// a grid of resident CTAs, and ONE atomic per CTA on the root counter: with
+// one per warp, 2^25 ids queued 2^20 atomics on that word and the pass took
+// 668 us; now 49 us (events around it; 128 MB: 2.7 TB/s).
+template <bool LABELS>
+__global__ void __launch_bounds__(256)
+k_validate(const int* __restrict__ a, int64_t n, int vec, DevState* __restrict__ ds) {
+    __shared__ int part[8];
+    int roots = 0;
+    bool bad = false;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
+    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; v0 < n; v0 += stride) {
+        int x[4];
+        if (vec && v0 + 4 <= n) {
+            const int4 q = *reinterpret_cast<const int4*>(a + v0);
+            x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; i++) x[i] = v0 + i < n ? a[v0 + i] : 0;  // past n: 0 <= 0, not counted
+        }
+        int y[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const bool in = x[i] >= 0 && (int64_t)x[i] <= v0 + i;
+            bad |= !in;
+            y[i] = LABELS && in && v0 + i < n && (int64_t)x[i] != v0 + i ? a[x[i]] : x[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            bad |= y[i] != x[i];
+            roots += v0 + i < n && (int64_t)x[i] == v0 + i;
+        }
     }
-    root = __reduce_add_sync(0xffffffffu, root);
-    if ((threadIdx.x & 31) == 0 && root) atomicAdd(&ds->roots, (unsigned long long)root);
+    if (bad) atomicOr(&ds->labels_bad, 1u);
+    roots = __reduce_add_sync(0xffffffffu, roots);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = roots;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < 8; w++) t += part[w];
+        if (t) atomicAdd(&ds->roots, (unsigned long long)t);
+    }
 }
 
-__global__ void __launch_bounds__(1024)
-k_validate_forest(const int* __restrict__ p, int64_t n, DevState* __restrict__ ds) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int root = 0;
-    if (v < n) {
-        const int x = p[v];
-        if (x < 0 || (int64_t)x > v) atomicOr(&ds->labels_bad, 1u);
-        root = (int64_t)x == v;
-    }
-    root = __reduce_add_sync(0xffffffffu, root);
-    if ((threadIdx.x & 31) == 0 && root) atomicAdd(&ds->roots, (unsigned long long)root);
-}
-
-cudaError_t launch_validate_forest(const int* p, int64_t n, DevState* ds, int block, cudaStream_t s) {
-    k_validate_forest<<<blocks_for(n, block), block, 0, s>>>(p, n, ds);
+template <bool LABELS>
+static cudaError_t validate(const int* a, int64_t n, DevState* ds, cudaStream_t s) {
+    int64_t g = (n + 1023) / 1024;
+    const int64_t cap = resident_grid<k_validate<LABELS>>(256);
+    if (g > cap) g = cap;
+    k_validate<LABELS><<<(unsigned)g, 256, 0, s>>>(a, n, pair_vec(a) == 2, ds);
     return cudaGetLastError();
 }
 
-cudaError_t launch_validate_labels(const int* lab, int64_t n, DevState* ds, int block,
-                                   cudaStream_t s) {
-    k_validate_labels<<<blocks_for(n, block), block, 0, s>>>(lab, n, ds);
-    return cudaGetLastError();
+cudaError_t launch_validate_forest(const int* p, int64_t n, DevState* ds, cudaStream_t s) {
+    return validate<false>(p, n, ds, s);
+}
+
+cudaError_t launch_validate_labels(const int* lab, int64_t n, DevState* ds, cudaStream_t s) {
+    return validate<true>(lab, n, ds, s);
 }
 
 }  // namespace cc
