@@ -121,7 +121,7 @@ typedef enum {
     CC_OPT_BULK_FIND = 15,       /* 1: Bulk-Query, and the relabel step of CC_OPT_UPDATE_SCHEDULE = 1,
                                     find all their roots with ONE Bulk-Find (Algorithm 4), whose
                                     path compression is shared by the whole minibatch (Theorem 3).
-                                    Synchronises once per tree level. Default 0 */
+                                    Default 0 */
     CC_OPT_QUERY_VARIANT = 16,   /* Bulk-Query kernel: 0 = one chunk of pairs per thread (default),
                                     1 = a persistent grid that loads the next chunk's pairs while
                                     working on the current one, 2 = warp-cooperative: a warp takes
@@ -484,14 +484,16 @@ cc_status cc_copy_nonloop(cc_ctx* ctx, int32_t* out, int64_t cap, int64_t* count
  * reported by cc_sync), with path compression shared by all of them:
  * afterwards every vertex on a path from some S[i] to its root points at that
  * root, and no other parent changes. Phase I walks up from all of S at once,
- * merging flows that meet; the Response Distributor (hashing into 3|R_u|
- * buckets and a counting sort, Section 4.1) lets Phase II hand each root back
- * down the recorded paths. `res`: device, k int32. Synchronises once per
- * level. */
+ * merging flows that meet; Phase II points every vertex met at its root.
+ * `res`: device, k int32 (it may be `S` itself). One cooperative kernel, or two
+ * kernels when the forest is known to be flat (right after a full compression,
+ * with no update since). Asynchronous, but for the scratch (12 bytes per vertex
+ * of the largest S so far) allocated on first use and grown. */
 cc_status cc_bulk_find(cc_ctx* ctx, const int32_t* S, int64_t k, int32_t* res);
 
 /* For the last Bulk-Find: the number of traversed non-root vertices
- * (|R_u| without R_0), and the number of Phase I and Phase II levels. */
+ * (|R_u| without R_0), and the number of Phase I and Phase II levels.
+ * Synchronises. */
 cc_status cc_bulk_find_stats(cc_ctx* ctx, int64_t* traversed, int32_t* levels_up,
                              int32_t* levels_down);
 

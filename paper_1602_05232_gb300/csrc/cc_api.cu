@@ -443,7 +443,8 @@ cc_status paper_update(cc_ctx* c, const int32_t* edges, int64_t k) {
             c->bf.res = q;
             c->bf.cap_res = 2 * k;
         }
-        e = cc::bulk_find(c->bf, c->parent, (int)c->n, edges, 2 * k, c->bf.res, c->ds, c->stream);
+        e = cc::bulk_find(c->bf, c->parent, (int)c->n, edges, 2 * k, c->bf.res, c->ds, c->flat,
+                          c->opt[CC_OPT_PDL] != 0, c->stream);
         c->launches[CC_K_UPDATE] += c->bf.launches - before;
         if (e != cudaSuccess) return cuda_fail(e, "schedule 1: Bulk-Find relabel");
     }
@@ -717,7 +718,8 @@ cc_status cc_bulk_query(cc_ctx* c, const int32_t* pairs, int64_t k, uint8_t* out
     if (c->opt[CC_OPT_BULK_FIND] == 1) {
         const uint64_t before = c->bf.launches;
         s = run(c, CC_K_QUERY, "bulk_query(Bulk-Find)", [&] {
-            return cc::bulk_find_query(c->bf, c->parent, (int)c->n, pairs, k, out, c->ds, c->stream);
+            return cc::bulk_find_query(c->bf, c->parent, (int)c->n, pairs, k, out, c->ds, c->flat,
+                                       c->opt[CC_OPT_PDL] != 0, c->stream);
         });
         c->launches[CC_K_QUERY] += c->bf.launches - before - 1;  // run() counted one
         return s;
@@ -1259,7 +1261,8 @@ cc_status cc_bulk_find(cc_ctx* c, const int32_t* S, int64_t k, int32_t* res) {
         return fail(CC_ERR_ARG, "cc_bulk_find: arrays must be 4-byte aligned");
     CC_DEVICE(c);
     const uint64_t before = c->bf.launches;
-    cudaError_t e = cc::bulk_find(c->bf, c->parent, (int)c->n, S, k, res, c->ds, c->stream);
+    cudaError_t e = cc::bulk_find(c->bf, c->parent, (int)c->n, S, k, res, c->ds, c->flat,
+                                  c->opt[CC_OPT_PDL] != 0, c->stream);
     c->launches[CC_K_QUERY] += c->bf.launches - before;
     if (e != cudaSuccess) return cuda_fail(e, "cc_bulk_find");
     return CC_OK;
@@ -1267,9 +1270,17 @@ cc_status cc_bulk_find(cc_ctx* c, const int32_t* S, int64_t k, int32_t* res) {
 
 cc_status cc_bulk_find_stats(cc_ctx* c, int64_t* traversed, int32_t* levels_up, int32_t* levels_down) {
     CC_CHECK_CTX(c);
-    if (traversed) *traversed = c->bf.traversed;
-    if (levels_up) *levels_up = c->bf.levels_up;
-    if (levels_down) *levels_down = c->bf.levels_down;
+    cc::BulkFindCounters h = {};
+    if (c->bf.count) {
+        CC_DEVICE(c);
+        cudaError_t e = cudaMemcpyAsync(&h, c->bf.count, sizeof h, cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "cc_bulk_find_stats");
+    }
+    const cc::BulkFindCounters::Stats& st = h.stats[c->bf.epoch & 1];
+    if (traversed) *traversed = (int64_t)st.traversed;
+    if (levels_up) *levels_up = (int32_t)st.levels;
+    if (levels_down) *levels_down = st.traversed ? (int32_t)st.depth + 1 : 0;
     return CC_OK;
 }
 

@@ -10,7 +10,7 @@ namespace cc {
 // atomicAdd per block on `count` (rather than one per warp): a list that
 // grows by a million items per launch through a single counter otherwise
 // queues tens of thousands of atomics on that one word. The warps' counts are
-// scanned in shared memory by one thread, which takes the block's range.
+// scanned by the first warp, which takes the block's range.
 // Every thread of the block must call it (it contains barriers); threads with
 // has == false get a slot they must not use. A warp reads and writes only its
 // own count, the next call's write coming after that call's warp-wide ballot
@@ -24,15 +24,17 @@ __device__ __forceinline__ unsigned block_slot(bool has, unsigned* __restrict__ 
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (lane == 0) warp_base[w] = __popc(mask);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned total = 0;
+    if (w == 0) {  // exclusive scan of the warps' counts; one lane takes the block's range
         const int warps = (blockDim.x + 31) >> 5;
-        for (int j = 0; j < warps; j++) {
-            const unsigned c = warp_base[j];
-            warp_base[j] = total;
-            total += c;
+        const unsigned own = lane < warps ? warp_base[lane] : 0u;
+        unsigned incl = own;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
         }
-        block_base = total ? atomicAdd(count, total) : 0u;
+        if (lane < warps) warp_base[lane] = incl - own;
+        if (lane == 31) block_base = incl ? atomicAdd(count, incl) : 0u;
     }
     __syncthreads();
     return block_base + warp_base[w] + __popc(mask & ((1u << lane) - 1));

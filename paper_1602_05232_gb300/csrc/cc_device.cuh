@@ -18,6 +18,14 @@
 
 namespace cc {
 
+// Programmatic dependent launch, device side. pdl_trigger: the kernel launched
+// after this one on the stream may start placing its CTAs (it still waits in
+// pdl_wait before touching results). pdl_wait: returns once the kernel before
+// this one has completed and its writes are visible; immediately when this
+// kernel was not launched as a dependent.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 __device__ __forceinline__ void flag(DevState* ds, unsigned bit) { atomicOr(&ds->status, bit); }
 
 __device__ __forceinline__ bool in_range(int x, int n) { return (unsigned)x < (unsigned)n; }

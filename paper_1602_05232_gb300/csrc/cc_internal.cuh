@@ -61,6 +61,65 @@ struct BigArgs {
     const int* alt = nullptr;
 };
 
+// A persistent grid for KERNEL at `block` threads (no dynamic shared memory):
+// resident CTAs per SM x SMs of the current device. Cached per host thread,
+// device and block size, so neither threads nor different GPUs share an entry.
+template <auto KERNEL>
+static int resident_grid(int block) {
+    thread_local int cache[16][33] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    int* slot = (dev >= 0 && dev < 16 && block > 0 && block <= 1024) ? &cache[dev][block / 32] : nullptr;
+    if (slot && *slot) return *slot;
+    int per_sm = 0, sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, block, 0);
+    const int c = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+    if (slot) *slot = c;
+    return c;
+}
+
+// Launch with per-launch attributes that apply to this kernel only (the
+// stream is left as it is): an optional L2 access-policy window, and
+// programmatic dependent launch, which lets the kernel's CTAs become resident
+// while the kernel before it on the stream drains; the kernel then waits for
+// that one in pdl_wait() (griddepcontrol.wait). A kernel that does not execute
+// the wait must not be launched with pdl.
+template <typename... Params, typename... Args>
+static void launch_windowed_smem(void (*kernel)(Params...), unsigned grid, int block, size_t smem, cudaStream_t s,
+                                 const cudaAccessPolicyWindow* window, bool pdl, Args... args) {
+    if (!window && !pdl) {
+        kernel<<<grid, block, smem, s>>>(args...);
+        return;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    unsigned na = 0;
+    if (window) {
+        attr[na].id = cudaLaunchAttributeAccessPolicyWindow;
+        attr[na].val.accessPolicyWindow = *window;
+        na++;
+    }
+    if (pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        na++;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... Params, typename... Args>
+static void launch_windowed(void (*kernel)(Params...), unsigned grid, int block, cudaStream_t s,
+                            const cudaAccessPolicyWindow* window, bool pdl, Args... args) {
+    launch_windowed_smem(kernel, grid, block, 0, s, window, pdl, args...);
+}
+
 // Alignment class of a pair array: 2 = 16-byte, 1 = 8-byte, 0 = 4-byte.
 int pair_vec(const void* p);
 
@@ -193,47 +252,40 @@ cudaError_t launch_compress_generic(int* parent, int64_t n, int* labels_out, int
 cudaError_t launch_depth(const int* parent, int64_t n, unsigned* max_depth,
                          unsigned long long* sum_depth, DevState* ds, cudaStream_t s);
 
-// ---- Bulk-Find (Algorithm 4) with the Response Distributor ----
+// ---- Bulk-Find (Algorithm 4) ----
+
+struct BulkFindCounters {        // on the device
+    struct Stats {
+        unsigned long long traversed;  // |R_u| without R_0
+        unsigned levels;               // Phase I levels
+        unsigned depth;                // longest path: Phase II has depth + 1 levels
+    } stats[2];                        // of the last call (epoch & 1); all zero for the next
+    unsigned front[3];                 // frontier sizes, zero between calls
+};
 
 struct BulkFindState {
     int* mark = nullptr;         // n entries: epoch stamp = visited in this call
     int epoch = 0;
     int* front[2] = {nullptr, nullptr};
     int* roots = nullptr;
-    int* D[2] = {nullptr, nullptr};  // Phase II frontiers of (v, root) pairs
-    int64_t cap_front = 0;           // entries of front/roots, pairs of D
-    int* R = nullptr;                // R_u: (from, to) pairs
-    int64_t cap_R = 0;
-    int* sorted = nullptr;           // R_u sorted by bucket
-    int64_t cap_R2 = 0;
-    int* bucket = nullptr;           // rho + 1 bucket offsets
-    int* cursor = nullptr;
-    int64_t cap_bucket = 0;
-    int* scan = nullptr;
-    int64_t cap_scan = 0;
-    int* work = nullptr;             // Phase II: bucket sizes, then their prefix sums
-    int64_t cap_work = 0;
-    int* res = nullptr;              // roots of the query endpoints (Bulk-Query)
+    int64_t cap_front = 0;           // entries of front and roots
+    int* res = nullptr;              // roots of the endpoints (relabel step of the paper's schedule)
     int64_t cap_res = 0;
-    unsigned* count = nullptr;
-    // statistics of the last call
-    int64_t traversed = 0;           // |R_u| without R_0
-    int32_t levels_up = 0, levels_down = 0;
+    BulkFindCounters* count = nullptr;
+    bool dirty = false;              // a failed launch may have left the counters non-zero
     uint64_t launches = 0;           // kernels launched, cumulative
 };
 
 // res[i] = root of S[i] (-1 for an id outside [0, n)); every node on the
-// paths from S to the roots points at its root afterwards. Synchronises once
-// per level.
+// paths from S to the roots points at its root afterwards. flat: every tree is
+// known to have height <= 1. pdl: programmatic dependent launch where a plain
+// launch does. Asynchronous, but for the allocations of a larger S than before.
 cudaError_t bulk_find(BulkFindState& b, int* parent, int n, const int* S, int64_t k, int* res,
-                      DevState* ds, cudaStream_t s);
+                      DevState* ds, bool flat, bool pdl, cudaStream_t s);
 // Bulk-Query through one Bulk-Find over all 2k endpoints.
 cudaError_t bulk_find_query(BulkFindState& b, int* parent, int n, const int* pairs, int64_t k,
-                            uint8_t* out, DevState* ds, cudaStream_t s);
+                            uint8_t* out, DevState* ds, bool flat, bool pdl, cudaStream_t s);
 void bulk_find_free(BulkFindState& b);
-// In-place exclusive scan of len ints; scratch needs scan_scratch_ints(len) ints.
-int64_t scan_scratch_ints(int64_t len);
-cudaError_t exclusive_scan(int* a, int64_t len, int* scratch, cudaStream_t s);
 
 // A'' from the roots found by a Bulk-Find over the 2k endpoints (res): the
 // pairs whose roots differ, with their component entries initialised.

@@ -15,66 +15,6 @@ static inline unsigned blocks_for(int64_t work, int64_t per_block) {
     return (unsigned)((work + per_block - 1) / per_block);
 }
 
-// Launch with per-launch attributes that apply to this kernel only (the
-// stream is left as it is): an optional L2 access-policy window, and
-// programmatic dependent launch, which lets the kernel's CTAs become resident
-// while the kernel before it on the stream drains; the kernel then waits for
-// that one in pdl_wait() (griddepcontrol.wait).
-template <typename... Params, typename... Args>
-static void launch_windowed(void (*kernel)(Params...), unsigned grid, int block, cudaStream_t s,
-                            const cudaAccessPolicyWindow* window, bool pdl, Args... args) {
-    if (!window && !pdl) {
-        kernel<<<grid, block, 0, s>>>(args...);
-        return;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    unsigned na = 0;
-    if (window) {
-        attr[na].id = cudaLaunchAttributeAccessPolicyWindow;
-        attr[na].val.accessPolicyWindow = *window;
-        na++;
-    }
-    if (pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        na++;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-// Programmatic dependent launch, device side. pdl_trigger: the kernel launched
-// after this one on the stream may start placing its CTAs (it still waits in
-// pdl_wait before touching results). pdl_wait: returns once the kernel before
-// this one has completed and its writes are visible; immediately when this
-// kernel was not launched as a dependent.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-
-// A persistent grid for KERNEL at `block` threads (no dynamic shared memory):
-// resident CTAs per SM x SMs of the current device. Cached per host thread,
-// device and block size, so neither threads nor different GPUs share an entry.
-template <auto KERNEL>
-static int resident_grid(int block) {
-    thread_local int cache[16][33] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int* slot = (dev >= 0 && dev < 16 && block > 0 && block <= 1024) ? &cache[dev][block / 32] : nullptr;
-    if (slot && *slot) return *slot;
-    int per_sm = 0, sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, block, 0);
-    const int c = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-    if (slot) *slot = c;
-    return c;
-}
-
 // ------------------------------------------------------------------ reset
 
 // parent[v] = v: n singletons, the empty graph G_0.
@@ -473,30 +413,8 @@ static void update_tiles_inst(const int* edges, int64_t k, int vec, int* parent,
     int64_t g = (k + (int64_t)E * block - 1) / ((int64_t)E * block);
     const int64_t cap = (int64_t)(per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
     if (g > cap) g = cap;
-    if (!window && !pdl) {
-        k_update_tiles<E><<<(unsigned)g, block, smem, s>>>(parent, n, edges, k, vec, ds, 0, minhook, fb);
-        return;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)g);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    unsigned na = 0;
-    if (window) {
-        attr[na].id = cudaLaunchAttributeAccessPolicyWindow;
-        attr[na].val.accessPolicyWindow = *window;
-        na++;
-    }
-    if (pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        na++;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    cudaLaunchKernelEx(&cfg, k_update_tiles<E>, parent, n, edges, k, vec, ds, (int)(pdl == 2), minhook, fb);
+    launch_windowed_smem(k_update_tiles<E>, (unsigned)g, block, smem, s, window, pdl != 0, parent, n, edges, k, vec, ds,
+                         (int)(pdl == 2), minhook, fb);
 }
 
 // --- VARIANT 4: filter pass + live-edge pass ------------------------------

@@ -41,9 +41,6 @@ constexpr int kOrderEpt = 8;                          // edges per thread per ti
 constexpr int kTile = kOrderBlock * kOrderEpt;        // 4096 edges
 constexpr int kMaxBuckets = 1 << 9;  // shared memory of the scatter kernel stays below 48 KiB
 
-__device__ __forceinline__ void pdl_trigger_o() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait_o() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-
 __device__ __forceinline__ int order_key(int u, int v, int n, int shift) {
     if (!(in_range(u, n) && in_range(v, n))) return 0;
     return (u < v ? u : v) >> shift;
@@ -90,12 +87,12 @@ __global__ void __launch_bounds__(kOrderBlock)
 k_order_count(const int* __restrict__ edges, int64_t k, int vec, int n, int shift, int nb,
               int* __restrict__ totals, int early, const unsigned* big, const DevState* ds) {
     __shared__ int hist[kMaxBuckets];
-    pdl_trigger_o();
+    pdl_trigger();
     if (big && ds->big_root >= 0) {  // the update reads the caller's order (BigArgs)
-        pdl_wait_o();                // still complete only after the kernel before
+        pdl_wait();                // still complete only after the kernel before
         return;
     }
-    if (!early) pdl_wait_o();
+    if (!early) pdl_wait();
     for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0;
     __syncthreads();
     const int64_t tiles = (k + kTile - 1) / kTile;
@@ -108,7 +105,7 @@ k_order_count(const int* __restrict__ edges, int64_t k, int vec, int n, int shif
         for (int i = 0; i < kOrderEpt; i++)
             if (e0 + i < k) atomicAdd(&hist[order_key(u[i], v[i], n, shift)], 1);
     }
-    if (early) pdl_wait_o();
+    if (early) pdl_wait();
     __syncthreads();
     for (int b = threadIdx.x; b < nb; b += blockDim.x)
         if (hist[b]) atomicAdd(&totals[b], hist[b]);
@@ -125,8 +122,8 @@ k_order_scatter(const int* __restrict__ edges, int64_t k, int vec, int n, int sh
     __shared__ unsigned short skey[kTile];
     __shared__ int warp_sums[kOrderBlock / 32];
     __shared__ bool last;
-    pdl_trigger_o();
-    pdl_wait_o();  // totals are complete
+    pdl_trigger();
+    pdl_wait();  // totals are complete
     if (big && ds->big_root >= 0) return;  // as in k_order_count: nothing was counted
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
         start[b] = totals[b];
@@ -188,20 +185,6 @@ k_order_scatter(const int* __restrict__ edges, int64_t k, int vec, int n, int sh
     }
 }
 
-template <typename K, typename... Args>
-cudaError_t launch_pdl(K kernel, unsigned grid, cudaStream_t s, bool pdl, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kOrderBlock);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 int order_grid(int64_t k) {
     static thread_local int cache[16] = {};
     int dev = 0;
@@ -246,13 +229,14 @@ cudaError_t launch_order_edges(const int* edges, int64_t k, int n, int log_bucke
     // The count kernel becomes a dependent launch only when it reads its
     // edges before the wait (pdl 2): launched early just to wait, its CTAs
     // would hold SM slots that the previous kernel's remaining CTAs need.
-    cudaError_t e = launch_pdl(k_order_count, (unsigned)G, s, pdl == 2, edges, k, vec, n, shift, nb, totals,
-                               (int)(pdl == 2), big, ds);
+    launch_windowed(k_order_count, (unsigned)G, kOrderBlock, s, nullptr, pdl == 2, edges, k, vec, n, shift, nb, totals,
+                    (int)(pdl == 2), big, ds);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_order_scatter, (unsigned)G, s, pdl != 0, edges, k, vec, n, shift, nb, totals, fill, done,
-                   reinterpret_cast<int2*>(out), big, ds);
+    launch_windowed(k_order_scatter, (unsigned)G, kOrderBlock, s, nullptr, pdl != 0, edges, k, vec, n, shift, nb, totals,
+                    fill, done, reinterpret_cast<int2*>(out), big, ds);
     *kernels = 2;
-    return e;
+    return cudaGetLastError();
 }
 
 }  // namespace cc

@@ -63,3 +63,62 @@ def test_validation_counts_roots_and_finds_each_fault(cc, n, shift):
             with pytest.raises(cc.CCError):
                 f.load_labels(dev(chain, shift))
             f.load_forest(dev(chain, shift))
+
+
+# ------------------------------------------------------------------ Bulk-Find
+
+def levels_up(par, S):
+    """Phase I levels, as the frontiers of Algorithm 4 run."""
+    seen, front, count = set(S), set(S), 0
+    while front:
+        count += 1
+        front = {int(par[v]) for v in front if par[v] != v} - seen
+        seen |= front
+    return count
+
+
+@pytest.mark.parametrize("k", [1, 31, 511, 512, 513, 4096, 1_500_001])
+@pytest.mark.parametrize("shape", ["flat", "random", "chain"])
+def test_bulk_find_at_block_and_grid_edges(cc, k, shape):
+    import oracle
+    n = 5000 if shape != "random" else 60_001
+    r = np.random.default_rng(k)
+    par = np.arange(n, dtype=np.int32)
+    if shape == "flat":
+        par[1:] = np.where(r.random(n - 1) < 0.5, 0, par[1:])
+    elif shape == "chain":
+        par[1:] = np.arange(n - 1)
+        par[::700] = np.arange(0, n, 700)
+    else:
+        par[1:] = (r.random(n - 1) * np.arange(1, n)).astype(np.int32)
+    S = r.integers(0, n, size=k).astype(np.int32)
+    want_par, want_res, want_t = oracle.bulk_find(par, S)
+    f = cc.Forest(n)
+    for again in range(2):      # the counters and stamps of the first call must not show in the second
+        if shape == "flat" and again:
+            f.load_labels(dev(par))     # known to be flat: the kernels without frontiers
+        else:
+            f.load_forest(dev(par))
+        Sd = dev(S, shift=1)
+        res = f.bulk_find(Sd, Sd if again else None)    # the roots may replace S itself
+        assert np.array_equal(res.cpu().numpy(), want_res)
+        assert np.array_equal(f.parent().cpu().numpy(), want_par)
+        t, up, down = f.bulk_find_stats()
+        depth = np.zeros(n, dtype=np.int64)
+        for v in range(1, n):
+            depth[v] = 0 if par[v] == v else depth[par[v]] + 1
+        assert t == want_t and up == levels_up(par, S.tolist())
+        assert down == (int(depth[S].max()) + 1 if want_t else 0)
+        if again:                       # the same through Bulk-Query: S as pairs
+            f.set_option("bulk_find", 1)
+            m = k - k % 2
+            got = f.bulk_query(dev(S[:m], shift=1).view(-1, 2)).cpu().numpy()
+            assert np.array_equal(got, (want_res[0:m:2] == want_res[1:m:2]).astype(np.uint8))
+            f.set_option("bulk_find", 0)
+    f.sync()
+    S[0] = n                    # an id outside [0, n): no root, and reported
+    got = f.bulk_find(dev(S)).cpu().numpy()
+    assert got[0] == -1 and np.array_equal(got[1:], want_res[1:])
+    with pytest.raises(cc.CCError) as ex:
+        f.sync()
+    assert ex.value.status == cc.CC_ERR_RANGE
