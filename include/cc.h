@@ -72,10 +72,10 @@ typedef enum {
     CC_OPT_EDGES_PER_THREAD = 1, /* edges (or pairs) per thread in update and query: 1, 2 or 4 (default 2) */
     CC_OPT_COMPRESS_EVERY = 2,   /* cc_bulk_update compresses after every c-th call; 0 = never (default 1) */
     CC_OPT_COMPRESS_SCOPE = 3,   /* scope of that automatic compression: a cc_compress_scope (default ALL) */
-    CC_OPT_QUERY_HALVING = 4,    /* how Bulk-Query finds walk: 0 read-only, all walks of a thread in
-                                    lockstep (default); 1 path halving, one pair after the other;
-                                    2 path splitting, all walks in lockstep (1 and 2 write, which
-                                    shortens paths for later operations) */
+    CC_OPT_QUERY_HALVING = 4,    /* how Bulk-Query finds walk (all pairs of a thread in lockstep): 0
+                                    read-only (default); 1 and 2 path splitting: every node walked
+                                    over is repointed at its grandparent, which shortens paths for
+                                    later operations */
     CC_OPT_PROFILE = 5,          /* 1: time every kernel with CUDA events on the handle's stream */
     CC_OPT_UPDATE_VARIANT = 6,   /* Bulk-Update kernel: 0 per-edge walks, 1 lockstep walks of all
                                     endpoints of a thread, 2 = 1 on a persistent grid that prefetches
@@ -257,7 +257,7 @@ cc_status cc_bulk_update(cc_ctx* ctx, const int32_t* edges, int64_t k);
 /* Bulk-Query (Algorithm 1; Section 3.1): out[i] = 1 if pairs[2i] and
  * pairs[2i+1] are connected by the edges added so far, else 0. `pairs`:
  * device, 2k int32; `out`: device, k bytes, written by the kernel. A pair
- * (u, u) answers 1. Finds are read-only unless CC_OPT_QUERY_HALVING is 1;
+ * (u, u) answers 1. Finds are read-only unless CC_OPT_QUERY_HALVING is set;
  * when the forest is known to be flat (right after a full compression, with
  * no update since) each answer is the equality of the two parents.
  * Errors: CC_ERR_ARG; ids outside [0, n) answer 0 and are reported by cc_sync. */

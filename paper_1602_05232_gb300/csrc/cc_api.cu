@@ -733,8 +733,7 @@ cc_status cc_bulk_query(cc_ctx* c, const int32_t* pairs, int64_t k, uint8_t* out
         if (s == CC_OK && !flat) c->flat = false;
         return s;
     }
-    const int64_t qh = c->opt[CC_OPT_QUERY_HALVING];
-    const int mode = c->flat ? 2 : (qh == 2 ? 3 : qh == 1 ? 1 : 0);
+    const int mode = c->flat ? 2 : c->opt[CC_OPT_QUERY_HALVING] != 0 ? 1 : 0;
     s = run(c, CC_K_QUERY, "bulk_query", [&] {
         return cc::launch_query(c->parent, (int)c->n, pairs, k, out, c->ds, mode, cfg_of(c), c->stream);
     });

@@ -144,8 +144,8 @@ cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevSt
 cudaError_t launch_update_split(int* parent, int n, const int* edges, int64_t k, DevState* ds, Launch cfg,
                                 int4* live, unsigned* count, int sel, cudaStream_t s);
 
-// mode: 0 read-only finds, 1 finds with path halving, 2 flat forest (parent
-// equality decides), 3 lockstep finds with path splitting.
+// mode: 0 read-only finds, 1 finds with path splitting, 2 flat forest (the
+// parents decide).
 cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_t* out,
                          DevState* ds, int mode, Launch cfg, cudaStream_t s);
 

@@ -610,89 +610,128 @@ __device__ __forceinline__ void store_answers(uint8_t* __restrict__ out, int64_t
 // One chunk of Algorithm 1: the E pairs (u, v) of this thread, answers in a.
 // Returns whether a pair had an id outside [0, n). MODE as for k_query. With
 // a largest-component bitmap, a pair whose endpoints are both marked is
-// answered 1 from the bitmap alone: it reads no parent and walks nothing
-// (its first parents are set equal, which every MODE below answers with 1).
-template <int E, int MODE>
-__device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, int (&u)[E], int (&v)[E],
+// answered 1 from the bitmap alone: it reads no parent and walks nothing.
+//
+// A pair is walked from its larger node only. Ids fall along every path, so
+// a root that is larger than the other side's node cannot be that side's root:
+// the pair is answered 0 there, and the other side is not read any further
+// (not at all, where the larger endpoint is itself a root). Otherwise the
+// larger node is replaced by its parent; nodes that meet answer 1. Every node
+// is read at most once, and none that walking both sides up to a verified root
+// would not read too. The kernel is bound by those gathers (one line per clock
+// and SM from L2, 71 G/s from DRAM), so what is not read is what it gains:
+// reading both endpoints and walking both to their roots, a pass over the
+// R-MAT stream (n = 2^24, 128 x 2^20 pairs, no compression) took 4.25 ms and
+// now takes 3.89; the 8192 x 8192 grid (32 x 2^22 pairs) 8.48 and now 7.01.
+//  LAZY: the smaller endpoint's parent is read only once the larger one's has
+//        not decided the pair. Otherwise both are read at once, which is a
+//        dependent read less where the pairs are too few to hide it.
+template <int E, int MODE, bool LAZY>
+__device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, const int (&u)[E], const int (&v)[E],
                                             int64_t e0, int64_t k, uint8_t (&a)[E],
                                             DevState* __restrict__ ds, const unsigned* bits) {
-    bool ok[E];
+    int hi[E], lo[E];
+    bool act[E];
     bool bad = false;
 #pragma unroll
     for (int i = 0; i < E; i++) {
-        ok[i] = e0 + i < k;
-        if (ok[i] && !(in_range(u[i], n) && in_range(v[i], n))) {
-            ok[i] = false;
+        bool ok = e0 + i < k;
+        if (ok && !(in_range(u[i], n) && in_range(v[i], n))) {
+            ok = false;
             bad = true;
         }
-        if (!ok[i]) { u[i] = 0; v[i] = 0; }
+        a[i] = ok && u[i] == v[i];
+        act[i] = ok && u[i] != v[i];
+        hi[i] = u[i] > v[i] ? u[i] : v[i];
+        lo[i] = u[i] > v[i] ? v[i] : u[i];
     }
-    bool hit[E];
-#pragma unroll
-    for (int i = 0; i < E; i++) hit[i] = bits && ok[i] && big_member(bits, u[i]) && big_member(bits, v[i]);
-    int pu[E], pv[E];
-#pragma unroll
-    for (int i = 0; i < E; i++) {
-        if (hit[i]) {
-            pu[i] = pv[i] = u[i];
-        } else if (MODE == 1 || MODE == 3) {
-            pu[i] = parent[u[i]];
-            pv[i] = parent[v[i]];
-        } else {
-            pu[i] = __ldg(parent + u[i]);
-            pv[i] = __ldg(parent + v[i]);
-        }
-    }
-    if (MODE == 2) {
-#pragma unroll
-        for (int i = 0; i < E; i++) a[i] = (uint8_t)(ok[i] && pu[i] == pv[i]);
-    } else if (MODE == 1) {
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            if (!ok[i]) { a[i] = 0; continue; }
-            if (pu[i] == pv[i]) { a[i] = 1; continue; }
-            int ru = pu[i] == u[i] ? u[i] : find_from(parent, u[i], pu[i], ds);
-            int rv = pv[i] == v[i] ? v[i] : find_from(parent, v[i], pv[i], ds);
-            a[i] = (uint8_t)(ru == rv);
-        }
-    } else if (MODE == 3) {
-        // all 2E walks in lockstep with path splitting (they write)
-        int x[2 * E], p[2 * E];
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            const bool live = ok[i] && pu[i] != pv[i];
-            x[2 * i] = u[i];     p[2 * i] = live ? pu[i] : u[i];
-            x[2 * i + 1] = v[i]; p[2 * i + 1] = live ? pv[i] : v[i];
-        }
-        walk_split<2 * E>(parent, x, p, ds);
+    if (bits) {
 #pragma unroll
         for (int i = 0; i < E; i++)
-            a[i] = (uint8_t)(ok[i] && (pu[i] == pv[i] || x[2 * i] == x[2 * i + 1]));
-    } else {
-        // walk state: x = current node, p = its parent; done when p >= x
-        int x[2 * E], p[2 * E];
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            bool live = ok[i] && pu[i] != pv[i];
-            x[2 * i] = u[i];     p[2 * i] = live ? pu[i] : u[i];
-            x[2 * i + 1] = v[i]; p[2 * i + 1] = live ? pv[i] : v[i];
-        }
-        while (true) {
-            bool any = false;
-#pragma unroll
-            for (int c = 0; c < 2 * E; c++) {
-                if (p[c] < x[c]) {
-                    x[c] = p[c];
-                    p[c] = __ldg(parent + x[c]);
-                    any = true;
-                }
+            if (act[i] && big_member(bits, hi[i]) && big_member(bits, lo[i])) {
+                a[i] = 1;
+                act[i] = false;
             }
-            if (!any) break;
+    }
+    int p[E], q[E];
+    if constexpr (MODE == 2) {
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            p[i] = act[i] ? __ldg(parent + hi[i]) : 0;
+            if (!LAZY) q[i] = act[i] ? __ldg(parent + lo[i]) : 0;
+        }
+        if (LAZY) {
+#pragma unroll
+            for (int i = 0; i < E; i++)  // p > lo: lo's root is another; p == lo: lo is the root
+                q[i] = act[i] && p[i] < lo[i] ? __ldg(parent + lo[i]) : lo[i];
+        }
+#pragma unroll
+        for (int i = 0; i < E; i++)
+            if (act[i]) a[i] = p[i] == q[i];
+        return bad;
+    }
+    // the node below hi (lo) on its walk, which is repointed past it (MODE 1); -1 at the endpoint
+    int bhi[E], blo[E];
+#pragma unroll
+    for (int i = 0; i < E; i++) bhi[i] = blo[i] = -1;
+    if constexpr (!LAZY) {
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            p[i] = q[i] = 0;
+            if (!act[i]) continue;
+            p[i] = MODE == 1 ? parent[hi[i]] : __ldg(parent + hi[i]);
+            q[i] = MODE == 1 ? parent[lo[i]] : __ldg(parent + lo[i]);
         }
 #pragma unroll
         for (int i = 0; i < E; i++) {
-            if (p[2 * i] > x[2 * i] || p[2 * i + 1] > x[2 * i + 1]) flag(ds, ST_CORRUPT);
-            a[i] = (uint8_t)(ok[i] && (pu[i] == pv[i] || x[2 * i] == x[2 * i + 1]));
+            if (!act[i]) continue;
+            if (p[i] > hi[i] || q[i] > lo[i]) flag(ds, ST_CORRUPT);
+            a[i] = p[i] == q[i] || p[i] == lo[i];
+            // decided, or one of them is a root above the other side's node
+            if (a[i] || p[i] >= hi[i] || (q[i] >= lo[i] && p[i] < lo[i])) {
+                act[i] = false;
+                continue;
+            }
+            bhi[i] = hi[i];
+            blo[i] = q[i] < lo[i] ? lo[i] : -1;
+            const bool swap = p[i] < q[i];
+            hi[i] = swap ? q[i] : p[i];
+            lo[i] = swap ? p[i] : q[i];
+            const int t = bhi[i];
+            bhi[i] = swap ? blo[i] : t;
+            blo[i] = swap ? t : blo[i];
+        }
+    }
+    while (true) {
+        bool any = false;
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            p[i] = 0;
+            if (!act[i]) continue;
+            p[i] = MODE == 1 ? parent[hi[i]] : __ldg(parent + hi[i]);
+            any = true;
+        }
+        if (!any) break;
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            if (!act[i]) continue;
+            if (p[i] >= hi[i]) {  // a root above lo's id, or a broken invariant: not connected
+                if (p[i] > hi[i]) flag(ds, ST_CORRUPT);
+                act[i] = false;
+                continue;
+            }
+            if (MODE == 1 && bhi[i] >= 0) parent[bhi[i]] = p[i];  // splitting: skip a level
+            if (p[i] == lo[i]) {
+                a[i] = 1;
+                act[i] = false;
+                continue;
+            }
+            const bool swap = p[i] < lo[i];
+            const int below = hi[i];
+            hi[i] = swap ? lo[i] : p[i];
+            lo[i] = swap ? p[i] : lo[i];
+            bhi[i] = swap ? blo[i] : below;
+            blo[i] = swap ? below : blo[i];
         }
     }
     return bad;
@@ -700,17 +739,17 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, int
 
 // Algorithm 1 over E pairs per thread. Lanes of a warp own consecutive pairs,
 // so the pair loads (16 B per lane) and the answer stores (E bytes per lane)
-// are coalesced across the warp.
-//  MODE 0: read-only finds through the read-only data path; the 2E walks of a
-//          thread advance in lockstep so their loads overlap.
-//  MODE 1: finds with path halving, one pair after the other (they write, so
-//          ordinary loads).
-//  MODE 2: flat forest (every tree of height <= 1): parent equality decides.
-//  MODE 3: the 2E walks in lockstep with path splitting (they write).
+// are coalesced across the warp. The E walks of a thread advance in lockstep,
+// so their loads overlap.
+//  MODE 0: read-only finds through the read-only data path.
+//  MODE 1: finds with path splitting: every node walked over is repointed at
+//          its grandparent (they write, so ordinary loads).
+//  MODE 2: flat forest (every tree of height <= 1): the parents decide.
+// LAZY: see query_chunk.
 // PERSIST: a persistent grid that loads the next chunk's pairs before working
 // on the current one, so those loads overlap the parent reads.
 // early: as for k_update.
-template <int E, int MODE, bool PERSIST>
+template <int E, int MODE, bool PERSIST, bool LAZY>
 __global__ void __launch_bounds__(1024)
 k_query(int* __restrict__ parent, int n, const int* __restrict__ pairs, int64_t k, int vec,
         uint8_t* __restrict__ out, int ovec, DevState* __restrict__ ds, int early,
@@ -726,7 +765,7 @@ k_query(int* __restrict__ parent, int n, const int* __restrict__ pairs, int64_t 
     if (early) pdl_wait();
     const unsigned* bits = big_active(big, ds);
     if (!PERSIST) {
-        bad = query_chunk<E, MODE>(parent, n, u, v, e0, k, a, ds, bits);
+        bad = query_chunk<E, MODE, LAZY>(parent, n, u, v, e0, k, a, ds, bits);
         store_answers<E>(out, e0, k, ovec != 0, a);
     } else {
         const int64_t stride = (int64_t)gridDim.x * blockDim.x * E;
@@ -734,7 +773,7 @@ k_query(int* __restrict__ parent, int n, const int* __restrict__ pairs, int64_t 
             const int64_t nx = e0 + stride;
             int nu[E] = {}, nv[E] = {};
             if (nx < k) load_pairs<E>(pairs, nx, k, vec, nu, nv);
-            bad |= query_chunk<E, MODE>(parent, n, u, v, e0, k, a, ds, bits);
+            bad |= query_chunk<E, MODE, LAZY>(parent, n, u, v, e0, k, a, ds, bits);
             store_answers<E>(out, e0, k, ovec != 0, a);
 #pragma unroll
             for (int i = 0; i < E; i++) {
@@ -850,22 +889,22 @@ k_query_warp(const int* __restrict__ parent, int n, const int* __restrict__ pair
     if (corrupt) flag(ds, ST_CORRUPT);
 }
 
-template <int E, int MODE, bool PERSIST>
+template <int E, int MODE, bool PERSIST, bool LAZY>
 static void query_one(unsigned g, int block, const cudaAccessPolicyWindow* window, int pdl, cudaStream_t s,
                       int* parent, int n, const int* pairs, int64_t k, int vec, uint8_t* out, int ovec,
                       DevState* ds, const unsigned* big) {
     if (PERSIST) {
-        const int c = resident_grid<k_query<E, MODE, PERSIST>>(block);
+        const int c = resident_grid<k_query<E, MODE, PERSIST, LAZY>>(block);
         if (g > (unsigned)c) g = (unsigned)c;
     }
-    launch_windowed(k_query<E, MODE, PERSIST>, g, block, s, window, pdl != 0, parent, n, pairs, k, vec, out, ovec,
-                    ds, (int)(pdl == 2), big);
+    launch_windowed(k_query<E, MODE, PERSIST, LAZY>, g, block, s, window, pdl != 0, parent, n, pairs, k, vec, out,
+                    ovec, ds, (int)(pdl == 2), big);
 }
 
-template <int MODE>
+template <int MODE, bool LAZY>
 static void query_inst(unsigned g, Launch cfg, cudaStream_t s, int* parent, int n,
                        const int* pairs, int64_t k, int vec, uint8_t* out, int ovec, DevState* ds) {
-#define CC_Q(E, P) query_one<E, MODE, P>(g, cfg.block, cfg.window, cfg.pdl, s, parent, n, pairs, k, vec, out, ovec, ds, cfg.big)
+#define CC_Q(E, P) query_one<E, MODE, P, LAZY>(g, cfg.block, cfg.window, cfg.pdl, s, parent, n, pairs, k, vec, out, ovec, ds, cfg.big)
     const bool persist = cfg.query_variant == 1;
     switch (cfg.ept) {
         case 1: if (persist) CC_Q(1, true); else CC_Q(1, false); break;
@@ -874,6 +913,12 @@ static void query_inst(unsigned g, Launch cfg, cudaStream_t s, int* parent, int 
     }
 #undef CC_Q
 }
+
+// From this many pairs the second parent of a pair is read only if the first
+// does not decide it (LAZY of query_chunk). Always
+// lazy, 50,001 pairs on 10^6 vertices cost 0.1 us more a query; never lazy, the
+// R-MAT pass takes 4.23 instead of 3.89 ms and the grid 8.08 instead of 7.01.
+constexpr int64_t kLazyPairs = 1 << 17;
 
 cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_t* out,
                          DevState* ds, int mode, Launch cfg, cudaStream_t s) {
@@ -892,10 +937,14 @@ cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_
     const int vec = pair_vec(pairs);
     const int ovec = (reinterpret_cast<uintptr_t>(out) % cfg.ept) == 0;
     const unsigned g = blocks_for(k, (int64_t)cfg.ept * cfg.block);
-    if (mode == 2) query_inst<2>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds);
-    else if (mode == 1) query_inst<1>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds);
-    else if (mode == 3) query_inst<3>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds);
-    else query_inst<0>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds);
+#define CC_QM(M) if (k >= kLazyPairs) query_inst<M, true>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds); \
+                 else query_inst<M, false>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds)
+    switch (mode) {
+        case 2: CC_QM(2); break;
+        case 1: CC_QM(1); break;
+        default: CC_QM(0); break;
+    }
+#undef CC_QM
     return cudaGetLastError();
 }
 

@@ -122,3 +122,53 @@ def test_bulk_find_at_block_and_grid_edges(cc, k, shape):
     with pytest.raises(cc.CCError) as ex:
         f.sync()
     assert ex.value.status == cc.CC_ERR_RANGE
+
+
+# ----------------------------------------------------------------- Bulk-Query
+
+def roots_of(par):
+    r = par.copy()
+    while not np.array_equal(r[r], r):
+        r = r[r]
+    return r
+
+
+@pytest.mark.parametrize("shape", ["flat", "random", "chains", "singletons"])
+@pytest.mark.parametrize("k", [1, 3, (1 << 17) - 1, 1 << 17, (1 << 17) + 5])
+def test_query_walks_answer_as_the_roots_do(cc, k, shape):
+    """Both sides of the size rule (two parents read at once, or the larger
+    endpoint's first), every walk mode, on forests of several heights."""
+    n = 100_003
+    r = np.random.default_rng(k)
+    par = np.arange(n, dtype=np.int32)
+    if shape == "flat":
+        par[1:] = np.where(r.random(n - 1) < 0.6, r.integers(0, 3, n - 1), par[1:])
+        par[:3] = 0, 1, 2
+    elif shape == "random":
+        par[1:] = np.where(r.random(n - 1) < 0.9, (r.random(n - 1) * np.arange(1, n)).astype(np.int32), par[1:])
+    elif shape == "chains":
+        par[40:] = np.arange(n - 40)
+    root = roots_of(par)
+    q = r.integers(0, n, size=(k, 2)).astype(np.int32)
+    q[::7, 1] = q[::7, 0]
+    q[1::11, 1] = par[q[1::11, 0]]
+    q[2::11, 1] = root[q[2::11, 0]]
+    want = (root[q[:, 0]] == root[q[:, 1]]).astype(np.uint8)
+    for mode in (0, 1, 2):
+        for extra in ({}, {"query_pairs_per_thread": 1}, {"query_pairs_per_thread": 4, "query_variant": 1}):
+            f = cc.Forest(n, query_halving=mode, **extra)
+            if shape == "flat":
+                f.load_labels(dev(root))
+            else:
+                f.load_forest(dev(par))
+            for shift in (0, 1):
+                assert np.array_equal(f.bulk_query(dev(q, shift)).cpu().numpy(), want), (mode, extra)
+            got = f.parent().cpu().numpy()      # the walks may only have skipped levels
+            assert (got <= par).all() and np.array_equal(roots_of(got), root)
+            f.sync()
+            bad = q.copy()
+            bad[-1] = n, 0
+            got = f.bulk_query(dev(bad)).cpu().numpy()
+            assert got[-1] == 0 and np.array_equal(got[:-1], want[:-1])
+            with pytest.raises(cc.CCError):
+                f.sync()
