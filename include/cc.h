@@ -129,13 +129,14 @@ typedef enum {
                                     ballot hands the next pair of the chunk to every slot whose
                                     walk has finished (read-only walks whatever
                                     CC_OPT_QUERY_HALVING says) */
-    CC_OPT_PDL = 17,             /* programmatic dependent launch of the Bulk-Update and Bulk-Query
-                                    kernels: 0 = off; 1 = each may become resident while the kernel
-                                    before it on the stream drains, and waits for that kernel to
-                                    complete before it reads anything (results unchanged; default);
-                                    2 = as 1, but each thread's first pairs are read BEFORE that
-                                    wait -- only for pair arrays that the kernel launched just
-                                    before on the same stream does not write */
+    CC_OPT_PDL = 17,             /* programmatic dependent launch of the Bulk-Update, Bulk-Query,
+                                    compression, label and reset kernels: 0 = off; 1 = each may
+                                    become resident while the kernel before it on the stream
+                                    drains, and waits for that kernel to complete before it reads
+                                    anything (results unchanged; default); 2 = as 1, but each
+                                    thread of an update or query reads its first pairs BEFORE
+                                    that wait -- only for pair arrays that the kernel launched
+                                    just before on the same stream does not write */
     CC_OPT_QUERY_PAIRS_PER_THREAD = 18, /* pairs per thread of the Bulk-Query kernel: 1, 2 or 4;
                                     0 = as CC_OPT_EDGES_PER_THREAD (default) */
     CC_OPT_HOOK = 19,            /* how the fused Bulk-Update links two roots: 0 = compare-and-swap on

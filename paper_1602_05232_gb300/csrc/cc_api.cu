@@ -242,12 +242,12 @@ cc_status do_compress(cc_ctx* c, int scope, const int32_t* edges, int64_t k) {
         unsigned* big = c->opt[CC_OPT_BIG_FILTER] > 0 ? c->big : nullptr;
         if (big) {
             cc_status s = run(c, CC_K_BIG_PICK, "compress(all): largest-tree pick", [&] {
-                return cc::launch_big_pick(c->parent, c->n, (int)c->opt[CC_OPT_BIG_FILTER], c->ds, c->stream);
+                return cc::launch_big_pick(c->parent, c->n, (int)c->opt[CC_OPT_BIG_FILTER], c->ds, c->opt[CC_OPT_PDL] != 0, c->stream);
             });
             if (s != CC_OK) return s;
         }
         cc_status s = run(c, CC_K_COMPRESS_ALL, "compress(all)", [&] {
-            return cc::launch_compress_all(c->parent, c->n, nullptr, c->ds, (int)c->opt[CC_OPT_BLOCK], c->stream, big);
+            return cc::launch_compress_all(c->parent, c->n, nullptr, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream, big);
         });
         if (s == CC_OK) c->flat = true;
         return s;
@@ -566,8 +566,7 @@ cc_status cc_create(int64_t n, cc_ctx** out) {
                     "cc_create(%lld): %s", (long long)n, cudaGetErrorString(e));
     }
     e = cudaMemsetAsync(c->ds, 0, sizeof(cc::DevState), c->stream);
-    if (e == cudaSuccess) e = big_invalidate(c);
-    if (e == cudaSuccess) e = cc::launch_reset(c->parent, n, 256, c->stream);
+    if (e == cudaSuccess) e = cc::launch_reset(c->parent, n, c->ds, 256, false, c->stream);
     c->launches[CC_K_RESET]++;
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -646,11 +645,8 @@ cc_status cc_sync(cc_ctx* c) {
 cc_status cc_reset(cc_ctx* c) {
     CC_CHECK_CTX(c);
     CC_DEVICE(c);
-    cudaError_t e = cudaMemsetAsync(&c->ds->unions, 0, sizeof(unsigned long long), c->stream);
-    if (e == cudaSuccess) e = big_invalidate(c);
-    if (e != cudaSuccess) return cuda_fail(e, "cc_reset");
     cc_status s = run(c, CC_K_RESET, "reset", [&] {
-        return cc::launch_reset(c->parent, c->n, (int)c->opt[CC_OPT_BLOCK], c->stream);
+        return cc::launch_reset(c->parent, c->n, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream);
     });
     if (s == CC_OK) {
         c->flat = true;
@@ -771,7 +767,7 @@ cc_status cc_labels(cc_ctx* c, int32_t* out) {
         return s;
     }
     cc_status s = run(c, CC_K_LABELS, "labels", [&] {
-        return cc::launch_compress_all(c->parent, c->n, out, c->ds, (int)c->opt[CC_OPT_BLOCK], c->stream);
+        return cc::launch_compress_all(c->parent, c->n, out, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream);
     });
     if (s == CC_OK) c->flat = true;
     return s;

@@ -53,9 +53,11 @@ struct Launch {
 // edges are dropped before their parent reads, and ordering them no longer
 // pays: launch_order_edges given the same `big` then does nothing, and an
 // update kernel given the ordered copy reads the caller's edges, `alt`,
-// instead. Both decide from big_root, which only the pick kernel writes, and
-// a full compression pass, launched without programmatic dependence, always
-// follows the pick, so every later kernel reads its final value.
+// instead. Both decide from big_root, which they may read before their own
+// wait for the kernel before them. Only the pick kernel and the reset write it,
+// and neither these nor the full compression pass that always follows the pick
+// (and waits for it) has a trigger: whatever is launched after them starts when
+// their CTAs have exited, and reads the final value.
 struct BigArgs {
     const unsigned* big = nullptr;
     const int* alt = nullptr;
@@ -131,7 +133,8 @@ cudaStream_t ctx_stream(const cc_ctx* c);
 int ctx_device(const cc_ctx* c);
 int32_t ctx_graphs(const cc_ctx* c);
 
-cudaError_t launch_reset(int* parent, int64_t n, int block, cudaStream_t s);
+// n singletons; also clears ds->unions and turns the largest-component filter off.
+cudaError_t launch_reset(int* parent, int64_t n, DevState* ds, int block, bool pdl, cudaStream_t s);
 
 cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevState* ds,
                           Launch cfg, cudaStream_t s);
@@ -152,14 +155,14 @@ cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_
 // Full compression; also writes labels to `out` when it is not null. With
 // `big` (n bits, rounded up to whole 32-bit words), bit v is set to whether v's
 // root is ds->big_root (nothing is written while that is -1).
-cudaError_t launch_compress_all(int* parent, int64_t n, int* out, DevState* ds, int block,
+cudaError_t launch_compress_all(int* parent, int64_t n, int* out, DevState* ds, int block, bool pdl,
                                 cudaStream_t s, unsigned* big = nullptr);
 
 // The root of the largest tree, estimated from kBigSample vertices (read-only
 // walks): ds->big_root = that root if at least min_share of the sample reached
 // it, else -1. One CTA.
 constexpr int kBigSample = 1024;
-cudaError_t launch_big_pick(const int* parent, int64_t n, int min_share, DevState* ds, cudaStream_t s);
+cudaError_t launch_big_pick(const int* parent, int64_t n, int min_share, DevState* ds, bool pdl, cudaStream_t s);
 // ds->big_members += the set bits of words[0, nwords).
 cudaError_t launch_big_count(const unsigned* words, int64_t nwords, DevState* ds, cudaStream_t s);
 

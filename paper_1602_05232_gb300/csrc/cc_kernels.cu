@@ -17,8 +17,18 @@ static inline unsigned blocks_for(int64_t work, int64_t per_block) {
 
 // ------------------------------------------------------------------ reset
 
-// parent[v] = v: n singletons, the empty graph G_0.
-__global__ void k_reset(int* __restrict__ parent, int64_t n) {
+// parent[v] = v: n singletons, the empty graph G_0, with no links made and no
+// tree marked (DevState's unions and big_root, which the first CTA sets here:
+// as two memsets in front they were two more operations on the stream). Kernels
+// that are launched as dependents may read big_root before their own wait; they
+// start once all CTAs here have exited, the first one after its write is visible.
+__global__ void k_reset(int* __restrict__ parent, int64_t n, DevState* __restrict__ ds) {
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ds->unions = 0ull;
+        ds->big_root = -1;
+        __threadfence();
+    }
     int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (v0 + 4 <= n) {
         int x = (int)v0;
@@ -28,9 +38,9 @@ __global__ void k_reset(int* __restrict__ parent, int64_t n) {
     }
 }
 
-cudaError_t launch_reset(int* parent, int64_t n, int block, cudaStream_t s) {
+cudaError_t launch_reset(int* parent, int64_t n, DevState* ds, int block, bool pdl, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    k_reset<<<blocks_for(n, 4LL * block), block, 0, s>>>(parent, n);
+    launch_windowed(k_reset, blocks_for(n, 4LL * block), block, s, nullptr, pdl, parent, n, ds);
     return cudaGetLastError();
 }
 
@@ -960,10 +970,16 @@ cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_
 // consecutive vertices); every lane of a warp takes part, so threads past n
 // do not leave early. (Counting the marked vertices here, one atomic per warp
 // on one word, doubled the pass: launch_big_count does it on demand.)
+// As a dependent launch it starts while the update drains, where a plain launch
+// costs a boundary of about 2 us on each side (ragged minibatches on 10^6
+// vertices, three kernels a step: 1250 -> 1011 us for 104 steps). It has no
+// explicit trigger, so its own dependents start as its CTAs exit: with one after
+// the wait, the kernels that follow all came in at once to wait (1195 us).
 template <bool OUT, bool BIG>
 __global__ void __launch_bounds__(1024)
 k_compress_all(int* __restrict__ parent, int64_t n, int* __restrict__ out,
                DevState* __restrict__ ds, unsigned* __restrict__ big) {
+    pdl_wait();
     const int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (!BIG && v0 >= n) return;
     const bool full = v0 + 4 <= n;
@@ -1054,7 +1070,8 @@ cudaError_t launch_big_count(const unsigned* words, int64_t nwords, DevState* ds
 // one (the smaller id on a tie) becomes ds->big_root if at least min_share of
 // the sample reached it, else -1. One CTA of kBigSample threads.
 __global__ void __launch_bounds__(kBigSample)
-k_big_pick(const int* __restrict__ parent, int64_t n, int min_share, DevState* __restrict__ ds) {
+k_big_pick(const int* parent, int64_t n, int min_share, DevState* __restrict__ ds) {
+    pdl_wait();
     constexpr int kSlots = 2 * kBigSample;
     __shared__ int key[kSlots];
     __shared__ int cnt[kSlots];
@@ -1103,32 +1120,28 @@ k_big_pick(const int* __restrict__ parent, int64_t n, int min_share, DevState* _
     }
 }
 
-cudaError_t launch_big_pick(const int* parent, int64_t n, int min_share, DevState* ds, cudaStream_t s) {
+cudaError_t launch_big_pick(const int* parent, int64_t n, int min_share, DevState* ds, bool pdl, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    k_big_pick<<<1, kBigSample, 0, s>>>(parent, n, min_share, ds);
+    launch_windowed(k_big_pick, 1u, kBigSample, s, nullptr, pdl, parent, n, min_share, ds);
     return cudaGetLastError();
 }
 
-cudaError_t launch_compress_all(int* parent, int64_t n, int* out, DevState* ds, int block,
+cudaError_t launch_compress_all(int* parent, int64_t n, int* out, DevState* ds, int block, bool pdl,
                                 cudaStream_t s, unsigned* big) {
     const unsigned g = blocks_for(n, 4LL * block);
-    const bool aligned_out = out && reinterpret_cast<uintptr_t>(out) % 16 == 0;
-    if (out && !aligned_out) {
-        // labels into a buffer without 16-byte alignment: compress, then copy
-        if (big) k_compress_all<false, true><<<g, block, 0, s>>>(parent, n, nullptr, ds, big);
-        else k_compress_all<false, false><<<g, block, 0, s>>>(parent, n, nullptr, ds, nullptr);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        return cudaMemcpyAsync(out, parent, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, s);
-    }
-    if (out) {
-        if (big) k_compress_all<true, true><<<g, block, 0, s>>>(parent, n, out, ds, big);
-        else k_compress_all<true, false><<<g, block, 0, s>>>(parent, n, out, ds, nullptr);
+    // labels into a buffer without 16-byte alignment: compress, then copy
+    int* direct = reinterpret_cast<uintptr_t>(out) % 16 == 0 ? out : nullptr;
+    if (direct) {
+        if (big) launch_windowed(k_compress_all<true, true>, g, block, s, nullptr, pdl, parent, n, direct, ds, big);
+        else launch_windowed(k_compress_all<true, false>, g, block, s, nullptr, pdl, parent, n, direct, ds, big);
     } else {
-        if (big) k_compress_all<false, true><<<g, block, 0, s>>>(parent, n, nullptr, ds, big);
-        else k_compress_all<false, false><<<g, block, 0, s>>>(parent, n, nullptr, ds, nullptr);
+        if (big) launch_windowed(k_compress_all<false, true>, g, block, s, nullptr, pdl, parent, n, direct, ds, big);
+        else launch_windowed(k_compress_all<false, false>, g, block, s, nullptr, pdl, parent, n, direct, ds, big);
     }
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && out && !direct)
+        e = cudaMemcpyAsync(out, parent, (size_t)n * sizeof(int), cudaMemcpyDeviceToDevice, s);
+    return e;
 }
 
 // Section 5.1's pragmatic compression for the endpoints of an edge array:
@@ -1137,6 +1150,7 @@ template <int E>
 __global__ void __launch_bounds__(1024)
 k_compress_touched(int* __restrict__ parent, int n, const int* __restrict__ edges, int64_t k,
                    int vec, DevState* __restrict__ ds) {
+    pdl_wait();
     const int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * E;
     if (e0 >= k) return;
     int u[E], v[E];
@@ -1163,9 +1177,9 @@ cudaError_t launch_compress_touched(int* parent, int n, const int* edges, int64_
     const int vec = pair_vec(edges);
     const unsigned g = blocks_for(k, (int64_t)cfg.ept * cfg.block);
     switch (cfg.ept) {
-        case 1: k_compress_touched<1><<<g, cfg.block, 0, s>>>(parent, n, edges, k, vec, ds); break;
-        case 2: k_compress_touched<2><<<g, cfg.block, 0, s>>>(parent, n, edges, k, vec, ds); break;
-        default: k_compress_touched<4><<<g, cfg.block, 0, s>>>(parent, n, edges, k, vec, ds); break;
+        case 1: launch_windowed(k_compress_touched<1>, g, cfg.block, s, nullptr, cfg.pdl != 0, parent, n, edges, k, vec, ds); break;
+        case 2: launch_windowed(k_compress_touched<2>, g, cfg.block, s, nullptr, cfg.pdl != 0, parent, n, edges, k, vec, ds); break;
+        default: launch_windowed(k_compress_touched<4>, g, cfg.block, s, nullptr, cfg.pdl != 0, parent, n, edges, k, vec, ds); break;
     }
     return cudaGetLastError();
 }

@@ -114,12 +114,13 @@ extern "C" cc_status cc_components_static(const int32_t* edges, int64_t k, int64
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cc::DevState* ds = reinterpret_cast<cc::DevState*>(scratch);
     int* parent = scratch + kHeaderInts;
-    const cc::Launch cfg{256, 2};
+    cc::Launch cfg{256, 2};
+    cfg.pdl = 1;
     // Start from n singletons with a clear status word, whatever the last call left.
     cudaError_t e = cudaMemsetAsync(ds, 0, sizeof(cc::DevState), s);
-    if (e == cudaSuccess) e = cc::launch_reset(parent, n, 256, s);
+    if (e == cudaSuccess) e = cc::launch_reset(parent, n, ds, 256, true, s);
     if (e == cudaSuccess) e = cc::launch_update(parent, (int)n, edges, k, ds, cfg, s);
-    if (e == cudaSuccess) e = cc::launch_compress_all(parent, n, labels, ds, 256, s);
+    if (e == cudaSuccess) e = cc::launch_compress_all(parent, n, labels, ds, 256, true, s);
     if (e == cudaSuccess && status)
         e = cudaMemcpyAsync(status, &ds->status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess)
