@@ -36,6 +36,15 @@ __device__ __forceinline__ int pair_vec_dev(const void* p) {
     return (a % 16 == 0) ? 2 : (a % 8 == 0) ? 1 : 0;
 }
 
+// Repoints x (not a root) at its ancestor `to`, for finds that shorten paths as
+// they go. An atomicMin whose result is not used: it is done where the line
+// lives, while a plain store to a line that other SMs are reading costs far
+// more on this chip. Measured with 2^18 threads that each write one random word
+// and read another, per pair: 0.129 ns with a store and 0.0125 with this on 2^16
+// words, 0.035 and 0.0124 on 2^20, 0.022 and 0.0137 on 2^22, 0.035 and 0.032
+// on 2^26. It also never raises an entry that another walk has lowered further.
+__device__ __forceinline__ void lower(int* parent, int x, int to) { atomicMin(parent + x, to); }
+
 // Root of x's tree, given p = parent[x] already read and p != x. Walks with
 // path halving: each visited node is repointed at its grandparent, which
 // roughly halves the path for later walks (the Section 5.1 idea of making
@@ -48,7 +57,7 @@ __device__ __forceinline__ int find_from(int* parent, int x, int p, DevState* ds
         }
         int gp = parent[p];
         if (gp == p) return p;
-        parent[x] = gp;
+        lower(parent, x, gp);
         x = gp;
         p = parent[x];
         if (p == x) return x;
@@ -218,7 +227,7 @@ __device__ __forceinline__ void walk_split(int* parent, int (&x)[W], int (&p)[W]
                     x[c] = p[c];
                     p[c] = x[c];
                 } else {
-                    parent[x[c]] = gp[c];  // splitting: skip a level
+                    lower(parent, x[c], gp[c]);  // splitting: skip a level
                     x[c] = p[c];
                     p[c] = gp[c];
                 }

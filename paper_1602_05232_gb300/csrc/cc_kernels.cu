@@ -730,7 +730,7 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, con
                 act[i] = false;
                 continue;
             }
-            if (MODE == 1 && bhi[i] >= 0) parent[bhi[i]] = p[i];  // splitting: skip a level
+            if (MODE == 1 && bhi[i] >= 0) lower(parent, bhi[i], p[i]);  // splitting: skip a level
             if (p[i] == lo[i]) {
                 a[i] = 1;
                 act[i] = false;
@@ -1164,7 +1164,7 @@ k_compress_touched(int* __restrict__ parent, int n, const int* __restrict__ edge
         if (p >= x) continue;
         const int r = walk_root(parent, x, p);
         while (p != r && p < x) {
-            parent[x] = r;
+            lower(parent, x, r);
             x = p;
             p = parent[x];
         }
