@@ -10,12 +10,12 @@
  *   Bulk-Query   answers, for each vertex pair of a minibatch, whether the two
  *                are connected by the edges added so far (Algorithm 1).
  *
- * Link rule. Hooking always makes the root with the larger id a child of the
- * root with the smaller id, so parent[v] <= v holds for every v at all times
- * and the root of each tree is the smallest id in its component. Section 3
- * links by size; any rule that joins two distinct roots is correct for
- * connectivity (the correctness lemma of Section 3.2 needs only that), and
- * this one needs no sizes array and no locks.
+ * Link rule. Hooking makes a root a child of a node of another tree with a
+ * smaller id, so parent[v] <= v holds for every v at all times and the root of
+ * each tree is the smallest id in its component. Section 3 links by size; any
+ * rule that joins two distinct trees at a root is correct for connectivity (the
+ * correctness lemma of Section 3.2 needs only that), and this one needs no
+ * sizes array and no locks.
  *
  * Conventions for every entry point:
  *  - Vertex ids are int32 in [0, n). An edge or a query pair is two int32s,
@@ -77,9 +77,8 @@ typedef enum {
                                     over is repointed at its grandparent, which shortens paths for
                                     later operations */
     CC_OPT_PROFILE = 5,          /* 1: time every kernel with CUDA events on the handle's stream */
-    CC_OPT_UPDATE_VARIANT = 6,   /* Bulk-Update kernel: 0 per-edge walks, 1 lockstep walks of all
-                                    endpoints of a thread, 2 = 1 on a persistent grid that prefetches
-                                    the next edges, 3 = 2 that also has the next chunk's first
+    CC_OPT_UPDATE_VARIANT = 6,   /* Bulk-Update kernel: 0 and 1 one chunk of edges per thread, 2 = 1
+                                    on a persistent grid that prefetches the next edges, 3 = 2 that also has the next chunk's first
                                     parent reads in flight during this chunk's walks, 4 = two
                                     kernels: a filter pass that reads every edge's first parents
                                     and lists the edges whose parents differ (16 B each; the list,
@@ -139,11 +138,11 @@ typedef enum {
                                     just before on the same stream does not write */
     CC_OPT_QUERY_PAIRS_PER_THREAD = 18, /* pairs per thread of the Bulk-Query kernel: 1, 2 or 4;
                                     0 = as CC_OPT_EDGES_PER_THREAD (default) */
-    CC_OPT_HOOK = 19,            /* how the fused Bulk-Update links two roots: 0 = compare-and-swap on
-                                    the larger root, retried from its new root on failure (default);
+    CC_OPT_HOOK = 19,            /* how the fused Bulk-Update links: 0 = compare-and-swap on the larger
+                                    root, going on from its new parent on failure (default);
                                     1 = atomicMin on the larger root's parent word, and when that
                                     word was no longer the root's own id, a join of the displaced
-                                    parent with the smaller root (cheaper when many edges of a
+                                    parent with the smaller node (cheaper when many edges of a
                                     minibatch hook onto one root); 2 = as 1 for the first
                                     Bulk-Update after cc_create or cc_reset (an empty forest,
                                     where hub vertices make that contention worst), as 0 after.
@@ -167,11 +166,10 @@ typedef enum {
                                     first use and grown with one stream synchronisation. Counted
                                     as CC_K_ORDER launches (two per ordered minibatch; they return
                                     at once while CC_OPT_BIG_FILTER's bitmap is in use) */
-    CC_OPT_HOOK_WARP = 22,       /* 1 = the fused Bulk-Update's lockstep variants (CC_OPT_UPDATE_VARIANT
-                                    1..4) group the hooks of a warp by target root: one lane per
-                                    distinct target writes it (compare-and-swap or atomicMin, per
-                                    CC_OPT_HOOK), the others join their smaller root with the
-                                    winner's, so a root that many edges of a minibatch hook onto
+    CC_OPT_HOOK_WARP = 22,       /* 1 = the fused Bulk-Update (CC_OPT_UPDATE_VARIANT 1..4) groups the
+                                    hooks of a warp by target root: one lane per distinct target
+                                    writes it (compare-and-swap or atomicMin, per CC_OPT_HOOK), the
+                                    others join their smaller node with the winner's, so a root that many edges of a minibatch hook onto
                                     sees one atomic per warp instead of one per edge. 0 = every
                                     lane hooks on its own (default). Same answers and labels */
     CC_OPT_BIG_FILTER = 23,      /* largest-component filter (the large-component skip of Afforest,
@@ -242,11 +240,11 @@ cc_status cc_reset(cc_ctx* ctx);
 
 /* Bulk-Update (Algorithm 2; Section 3.2): add the k edges at `edges`
  * (device, 2k int32, u0 v0 u1 v1 ...) to the graph. One fused kernel: per
- * edge, find both roots with path halving (Algorithm 2's relabel step, with
- * the walk shortening of Section 5.1), drop it if the roots agree (the self-
- * loop filter of Algorithm 2), else hook the larger root under the smaller
- * with a compare-and-swap, re-finding and retrying when another edge moved
- * that root first. This replaces Algorithm 2's connected-components step and
+ * edge, read both parents and drop it if they agree (the self-loop filter of
+ * Algorithm 2), else move the larger of the two nodes up, shortening the paths
+ * passed (Algorithm 2's relabel step, with Section 5.1's compression), until
+ * the sides meet or it is a root, and hook that under the other side's node
+ * with a compare-and-swap, going on when another edge moved it first. This replaces Algorithm 2's connected-components step and
  * Parallel-Join (Algorithm 3): both only exist to join distinct roots without
  * conflicts. The order of edges inside a minibatch does not matter (Section
  * 2); self-loops and repeated edges are legal no-ops. k = 0 is a no-op. Then,

@@ -212,7 +212,7 @@ cc::Launch cfg_of(const cc_ctx* c) {
     return cc::Launch{(int)c->opt[CC_OPT_BLOCK], (int)c->opt[CC_OPT_EDGES_PER_THREAD],
                       (int)c->opt[CC_OPT_UPDATE_VARIANT], (int)c->opt[CC_OPT_QUERY_VARIANT],
                       c->window.num_bytes > 0 ? &c->window : nullptr, (int)c->opt[CC_OPT_PDL],
-                      (int)c->opt[CC_OPT_QUERY_PAIRS_PER_THREAD], (int)(c->opt[CC_OPT_HOOK] == 1),
+                      (int)c->opt[CC_OPT_QUERY_PAIRS_PER_THREAD], c->opt[CC_OPT_HOOK] == 1 ? cc::HOOK_MIN : 0,
                       (int)c->opt[CC_OPT_HOOK_WARP], c->opt[CC_OPT_BIG_FILTER] > 0 ? c->big : nullptr};
 }
 
@@ -258,11 +258,18 @@ cc_status do_compress(cc_ctx* c, int scope, const int32_t* edges, int64_t k) {
     });
 }
 
+// Whether a full compression follows the Bulk-Update about to run.
+bool compress_due(const cc_ctx* c) {
+    const int64_t every = c->opt[CC_OPT_COMPRESS_EVERY];
+    return every > 0 && (c->update_calls + 1) % (uint64_t)every == 0;
+}
+
 // Launch options of a Bulk-Update: CC_OPT_HOOK = 2 hooks with atomicMin only
 // for the first Bulk-Update on an empty forest (`first`), CAS afterwards.
 cc::Launch update_cfg(const cc_ctx* c, bool first) {
     cc::Launch cfg = cfg_of(c);
-    if (c->opt[CC_OPT_HOOK] == 2) cfg.minhook = first ? 1 : 0;
+    if (c->opt[CC_OPT_HOOK] == 2 && first) cfg.hook |= cc::HOOK_MIN;
+    if (!compress_due(c) || c->opt[CC_OPT_COMPRESS_SCOPE] != CC_COMPRESS_ALL) cfg.hook |= cc::HOOK_CLIMB;
     return cfg;
 }
 
@@ -670,6 +677,7 @@ cc_status cc_bulk_update(cc_ctx* c, const int32_t* edges, int64_t k) {
     if (by_size(c) && c->opt[CC_OPT_UPDATE_SCHEDULE] != 1)
         return fail(CC_ERR_UNSUPPORTED, "union by size (CC_OPT_LINK = 1) needs CC_OPT_UPDATE_SCHEDULE = 1");
     const bool first = c->fresh;  // the forest has no edge yet
+    const bool compress = compress_due(c);
     const int32_t* given = edges;
     const bool fused = c->opt[CC_OPT_UPDATE_SCHEDULE] != 1;
     // the fused kernels read the caller's edges instead of an ordered copy
@@ -698,8 +706,7 @@ cc_status cc_bulk_update(cc_ctx* c, const int32_t* edges, int64_t k) {
     if (s != CC_OK) return s;
     c->flat = false;
     c->update_calls++;
-    const int64_t every = c->opt[CC_OPT_COMPRESS_EVERY];
-    if (every > 0 && c->update_calls % (uint64_t)every == 0)
+    if (compress)
         return do_compress(c, (int)c->opt[CC_OPT_COMPRESS_SCOPE], given, k);  // a set: same endpoints
     return CC_OK;
 }

@@ -1,13 +1,13 @@
 // Device primitives of the union-find forest: find and hook.
 //
 // Forest invariant: parent[x] <= x for every x, with equality exactly at the
-// roots. Hooks link the larger root under the smaller, and path halving and
-// compression only repoint a node at one of its ancestors, so every write
-// keeps the invariant. Consequences used throughout:
+// roots. Hooks link a root under a smaller node of another tree, and path
+// shortening and compression only repoint a node at one of its ancestors, so
+// every write keeps the invariant. Consequences used throughout:
 //  * every walk strictly decreases the id, so it ends within n steps (no
 //    iteration limit is needed, and none can livelock);
 //  * once a node stops being a root it never becomes one again, so only roots
-//    are ever compare-and-swapped and only non-roots ever get plain stores;
+//    are ever linked and only non-roots are ever repointed;
 //  * a value read late or early is still an ancestor: two endpoints that reach
 //    the same node are connected, whatever else is happening.
 #pragma once
@@ -88,152 +88,6 @@ __device__ __forceinline__ int hook(int* parent, int ru, int rv, DevState* ds) {
         if (hi == ru) ru = r; else rv = r;
     }
     return 0;
-}
-
-// The same join with atomicMin instead of a compare-and-swap: parent[hi] is
-// lowered to lo (hi = the larger id). If hi was still a root, that is the
-// link. If not, its parent `old` comes back. When old > lo this call has just
-// moved hi's subtree from old's tree into lo's, and when old < lo it changed
-// nothing; either way the loop goes on joining old and lo, from their current
-// roots, which are both below hi -- so it ends, and old's tree is joined to
-// lo's, which keeps every earlier connection. Pointers only ever decrease, so
-// no cycle can form. A hook counts only a write at a root, so the number of
-// trees drops by exactly the links it returns. Under contention (many edges
-// of a minibatch on one hub root) every caller issues one atomic on the hub
-// and repairs elsewhere, where the CAS version fails, walks and retries in
-// rounds.
-static __device__ __noinline__ int hook_min(int* parent, int ru, int rv, DevState* ds) {
-    while (ru != rv) {
-        const int hi = ru > rv ? ru : rv;
-        const int lo = ru > rv ? rv : ru;
-        const int old = atomicMin(parent + hi, lo);
-        if (old == hi) return 1;
-        if (old > hi) {
-            flag(ds, ST_CORRUPT);
-            return 0;
-        }
-        if (old == lo) return 0;
-        ru = find_halving(parent, old, ds);
-        rv = find_halving(parent, lo, ds);
-    }
-    return 0;
-}
-
-// hook or hook_min, chosen per launch.
-__device__ __forceinline__ int hook_as(int* parent, int ru, int rv, DevState* ds, int minhook) {
-    return minhook ? hook_min(parent, ru, rv, ds) : hook(parent, ru, rv, ds);
-}
-
-// The hooks of a whole warp, grouped by target. Must be called by all 32
-// lanes together. Lane l joins roots-or-former-roots a[i], b[i] for every i
-// with want[i]. In each round the lanes whose larger root `hi` is the same
-// form a group (__match_any_sync): only one lane of the group -- the one
-// with the smallest `lo` -- writes parent[hi], with a compare-and-swap
-// (hook) or an atomicMin (hook_min), instead of every lane of the group
-// contending for that word. Then:
-//  - the write linked hi under lo_min: the leader is done, and every other
-//    member joins its own lo with lo_min (hi is now in lo_min's tree);
-//  - compare-and-swap failed (hi is no longer a root): the leader finds the
-//    root r of hi's new parent once, and every member continues with
-//    (r, its lo);
-//  - atomicMin found hi under old < hi: the leader continues joining old
-//    and lo_min (as hook_min does), every other member joins its lo with
-//    lo_min.
-// Every continuing pair has both ids below hi, so each lane's larger id
-// strictly decreases from round to round and the loop ends. Returns the
-// links this lane made (a write at a root counts once).
-template <int E>
-__device__ __forceinline__ int hook_warp(int* parent, const bool (&want0)[E], const int (&a0)[E],
-                                         const int (&b0)[E], DevState* ds, int minhook) {
-    const unsigned full = 0xffffffffu;
-    const int lane = (int)(threadIdx.x & 31u);
-    int made = 0;
-#pragma unroll
-    for (int i = 0; i < E; i++) {
-        bool want = want0[i];
-        int a = a0[i], b = b0[i];
-        while (__any_sync(full, want)) {
-            int hi = a > b ? a : b, lo = a > b ? b : a;
-            if (want && hi == lo) want = false;
-            const unsigned m = __match_any_sync(full, want ? hi : -1 - lane);
-            if (!want) continue;
-            const int lo_min = __reduce_min_sync(m, lo);
-            const int leader = __ffs(__ballot_sync(m, lo == lo_min)) - 1;
-            int old = 0;
-            if (lane == leader)
-                old = minhook ? atomicMin(parent + hi, lo_min) : atomicCAS(parent + hi, hi, lo_min);
-            old = __shfl_sync(m, old, leader);
-            if (old > hi) {  // broken invariant: stop rather than loop
-                if (lane == leader) flag(ds, ST_CORRUPT);
-                want = false;
-            } else if (old == hi) {  // linked hi under lo_min
-                if (lane == leader) {
-                    made++;
-                    want = false;
-                } else {
-                    a = lo;
-                    b = lo_min;
-                }
-            } else if (minhook) {  // hi was already under old
-                if (lane == leader) {
-                    if (old == lo_min) {
-                        want = false;
-                    } else {
-                        a = find_halving(parent, old, ds);
-                        b = find_halving(parent, lo_min, ds);
-                    }
-                } else {
-                    a = lo;
-                    b = lo_min;
-                }
-            } else {  // compare-and-swap failed: hi is no longer a root
-                int r = 0;
-                if (lane == leader) r = find_halving(parent, old, ds);
-                a = __shfl_sync(m, r, leader);
-                b = lo;
-            }
-        }
-    }
-    return made;
-}
-
-// Walk W chains to their roots in lockstep with path splitting. Chain c is at
-// node x[c] whose parent p[c] has been read; it is finished when p[c] >= x[c]
-// (p == x: x is the root). Each round reads the grandparent of every
-// unfinished chain -- independent loads, all in flight together -- then
-// repoints the node at its grandparent and moves up one level. On exit x[c]
-// is the root of chain c (or, with a broken invariant, where it stopped).
-template <int W>
-__device__ __forceinline__ void walk_split(int* parent, int (&x)[W], int (&p)[W], DevState* ds) {
-    while (true) {
-        int gp[W];
-        bool any = false;
-#pragma unroll
-        for (int c = 0; c < W; c++) {
-            gp[c] = p[c];
-            if (p[c] < x[c]) {
-                gp[c] = parent[p[c]];
-                any = true;
-            }
-        }
-        if (!any) break;
-#pragma unroll
-        for (int c = 0; c < W; c++) {
-            if (p[c] < x[c]) {
-                if (gp[c] == p[c]) {
-                    x[c] = p[c];          // p is the root
-                } else if (gp[c] > p[c]) {
-                    flag(ds, ST_CORRUPT);
-                    x[c] = p[c];
-                    p[c] = x[c];
-                } else {
-                    lower(parent, x[c], gp[c]);  // splitting: skip a level
-                    x[c] = p[c];
-                    p[c] = gp[c];
-                }
-            }
-        }
-    }
 }
 
 // Largest-component filter (the large-component skip of Afforest: Sutton,

@@ -29,10 +29,16 @@ struct DevState {
     unsigned long long big_members;  // set bits of the bitmap (launch_big_count, on demand)
 };
 
+// How the fused Bulk-Update links two trees (see join_edges).
+enum : int {
+    HOOK_MIN = 1,    // with atomicMin and a repair instead of a compare-and-swap
+    HOOK_CLIMB = 2,  // under the other side's root, not just its node
+};
+
 struct Launch {
     int block;        // threads per block, multiple of 32
     int ept;          // edges (pairs) per thread: 1, 2 or 4
-    int variant = 0;  // update kernel: 0 per-edge walks, 1 lockstep walks, 2 persistent + prefetch,
+    int variant = 0;  // update kernel: 0 and 1 one chunk per thread, 2 persistent + prefetch,
                       // 3 persistent + two-stage prefetch (edges two chunks ahead, parents one),
                       // 4 filter pass + live-edge pass (launch_update_split),
                       // 5 persistent tiles whose open edges the whole CTA walks from a shared-memory list
@@ -40,8 +46,8 @@ struct Launch {
     const cudaAccessPolicyWindow* window = nullptr;  // L2 window over the forest, or none
     int pdl = 0;  // programmatic dependent launch: 0 off, 1 wait first, 2 first pairs before the wait
     int qept = 0; // pairs per thread of the query kernel (0 = ept)
-    int minhook = 0;  // 1: Bulk-Update hooks with atomicMin + repair (hook_min) instead of CAS
-    int warphook = 0; // 1: the hooks of a warp are grouped by target root (hook_warp); lockstep variants
+    int hook = 0;     // how Bulk-Update links (HOOK_*)
+    int warphook = 0; // 1: the link attempts of a warp are grouped by target root; variants 1..4
     const unsigned* big = nullptr;  // largest-component bitmap (n bits), or none: pairs whose two
                                     // endpoints are marked are answered / dropped without walks
     const int* alt = nullptr;       // Bulk-Update on an ordered copy: the caller's edges, which the

@@ -46,141 +46,6 @@ cudaError_t launch_reset(int* parent, int64_t n, DevState* ds, int block, bool p
 
 // ------------------------------------------------------------ Bulk-Update
 
-// One fused pass of Algorithm 2 over E edges: the first parent reads of both
-// endpoints of all E edges are issued together; equal parents mean the edge
-// joins a tree to itself and is dropped at once (the common case once trees
-// are flat, and the self-loop filter of Algorithm 2). The other endpoints are
-// walked to their roots -- VARIANT 0 one edge at a time with path halving,
-// VARIANTs 1 and 2 all 2E walks in lockstep with path splitting -- and the
-// roots are hooked. Returns the number of links made.
-template <int E, int VARIANT, bool WARP = false>
-__device__ __forceinline__ int update_edges(int* __restrict__ parent, int n,
-                                            const int (&u)[E], const int (&v)[E], int64_t e0,
-                                            int64_t k, DevState* __restrict__ ds, int minhook,
-                                            const unsigned* bits) {
-    bool ok[E];
-    bool bad = false;
-    int made = 0;
-#pragma unroll
-    for (int i = 0; i < E; i++) {
-        ok[i] = e0 + i < k;
-        if (ok[i] && !(in_range(u[i], n) && in_range(v[i], n))) {
-            ok[i] = false;
-            bad = true;
-        }
-    }
-    if (bad) flag(ds, ST_RANGE);
-    if (bits) {  // both endpoints in the marked tree: already joined
-#pragma unroll
-        for (int i = 0; i < E; i++)
-            if (ok[i] && big_member(bits, u[i]) && big_member(bits, v[i])) ok[i] = false;
-    }
-    if constexpr (VARIANT == 0) {
-        int pu[E], pv[E];
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            pu[i] = ok[i] ? parent[u[i]] : 0;
-            pv[i] = ok[i] ? parent[v[i]] : 0;
-        }
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            if (!ok[i] || pu[i] == pv[i]) continue;
-            int ru = pu[i] == u[i] ? u[i] : find_from(parent, u[i], pu[i], ds);
-            int rv = pv[i] == v[i] ? v[i] : find_from(parent, v[i], pv[i], ds);
-            made += hook_as(parent, ru, rv, ds, minhook);
-        }
-        return made;
-    } else {
-        // lockstep: chain c = 2i (u side) and 2i+1 (v side); finished when p >= x
-        int x[2 * E], p[2 * E];
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            x[2 * i] = ok[i] ? u[i] : 0;
-            x[2 * i + 1] = ok[i] ? v[i] : 0;
-        }
-#pragma unroll
-        for (int c = 0; c < 2 * E; c++) p[c] = ok[c / 2] ? parent[x[c]] : x[c];
-        bool live[E];
-#pragma unroll
-        for (int i = 0; i < E; i++) {
-            live[i] = ok[i] && p[2 * i] != p[2 * i + 1];
-            if (!live[i]) {  // nothing to walk for this edge
-                p[2 * i] = x[2 * i];
-                p[2 * i + 1] = x[2 * i + 1];
-            }
-        }
-        walk_split<2 * E>(parent, x, p, ds);
-        if constexpr (WARP) {  // every lane of the warp is here (see the kernels)
-            int a[E], b[E];
-#pragma unroll
-            for (int i = 0; i < E; i++) {
-                a[i] = x[2 * i];
-                b[i] = x[2 * i + 1];
-            }
-            made = hook_warp<E>(parent, live, a, b, ds, minhook);
-        } else {
-#pragma unroll
-            for (int i = 0; i < E; i++)
-                if (live[i]) made += hook_as(parent, x[2 * i], x[2 * i + 1], ds, minhook);
-        }
-        return made;
-    }
-}
-
-// early: the first edges are read before the wait for the previous kernel
-// (programmatic dependent launch; see launch_windowed), else after it.
-// warphook (lockstep variants only): the hooks of a warp are grouped by
-// target (hook_warp), so every lane of a warp that has any edge left goes
-// through each round of the loop, with no edges of its own if it has none.
-template <int E, int VARIANT, bool WARP>
-__global__ void __launch_bounds__(1024)
-k_update(int* __restrict__ parent, int n, const int* __restrict__ edges, int64_t k, int vec,
-         DevState* __restrict__ ds, int early, int minhook, BigArgs fb) {
-    pdl_trigger();
-    if (!early) pdl_wait();
-    if (fb.alt && big_active(fb.big, ds)) {  // the filter is on: the edges were not ordered
-        edges = fb.alt;
-        vec = pair_vec_dev(fb.alt);
-    }
-    int made = 0;
-    int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * E;
-    if (VARIANT < 2) {
-        // with warphook, every lane goes in if any lane of its warp has edges
-        bool warp_busy = false;
-        if constexpr (WARP) warp_busy = __any_sync(0xffffffffu, e0 < k);
-        if (e0 < k || warp_busy) {
-            int u[E], v[E];
-            load_pairs<E>(edges, e0, k, vec, u, v);
-            if (early) pdl_wait();
-            made = update_edges<E, VARIANT, WARP>(parent, n, u, v, e0, k, ds, minhook, big_active(fb.big, ds));
-        }
-    } else {
-        // persistent grid: loop over chunks, loading the next chunk's edges
-        // before walking the current one so their latency overlaps
-        const int64_t stride = (int64_t)gridDim.x * blockDim.x * E;
-        int u[E], v[E];
-        if (e0 < k) load_pairs<E>(edges, e0, k, vec, u, v);
-        if (early) pdl_wait();
-        const unsigned* bits = big_active(fb.big, ds);
-        while (WARP ? __any_sync(0xffffffffu, e0 < k) : e0 < k) {
-            const int64_t nx = e0 + stride;
-            int nu[E] = {}, nv[E] = {};
-            if (nx < k) load_pairs<E>(edges, nx, k, vec, nu, nv);
-            made += update_edges<E, 1, WARP>(parent, n, u, v, e0, k, ds, minhook, bits);
-#pragma unroll
-            for (int i = 0; i < E; i++) {
-                u[i] = nu[i];
-                v[i] = nv[i];
-            }
-            e0 = nx;
-        }
-    }
-    made = __reduce_add_sync(0xffffffffu, made);
-    if ((threadIdx.x & 31) == 0 && made) atomicAdd(&ds->unions, (unsigned long long)made);
-}
-
-// --- VARIANT 3: the persistent grid with a two-stage prefetch -------------
-
 // Bit i set when this thread's edge i at e0 exists and has both endpoints in
 // range, and (with a largest-component bitmap) they are not both marked;
 // range errors are flagged here, once per chunk.
@@ -196,7 +61,7 @@ __device__ __forceinline__ unsigned edge_mask(int n, const int (&u)[E], const in
         else bad = true;
     }
     if (bad) flag(ds, ST_RANGE);
-    if (bits) {
+    if (bits) {  // both endpoints in the marked tree: already joined
 #pragma unroll
         for (int i = 0; i < E; i++)
             if (((m >> i) & 1u) && big_member(bits, u[i]) && big_member(bits, v[i])) m &= ~(1u << i);
@@ -219,40 +84,192 @@ __device__ __forceinline__ void gather_parents(const int* parent, unsigned m, co
 
 // The rest of the fused pass for edges whose first parents pu, pv were read
 // earlier, possibly before other links of this minibatch: a parent read then
-// is still an ancestor now (links only put roots under roots, and splitting
-// only repoints a node at an ancestor), so walking on from it reaches the
-// current root, and equal values still prove the endpoints joined.
-template <int E, bool WARP = false>
-__device__ __forceinline__ int walk_and_hook(int* parent, unsigned m, const int (&u)[E], const int (&v)[E],
-                                             const int (&pu)[E], const int (&pv)[E], DevState* ds,
-                                             int minhook) {
-    int x[2 * E], p[2 * E];
-    bool live[E];
+// is still an ancestor now (links only put roots under other trees' nodes, and
+// splitting only repoints a node at an ancestor), so going on from it reaches
+// the current root, and equal values still prove the endpoints joined.
+//
+// Each edge is two nodes, one of either side, and the larger one is moved up
+// until the sides meet or it is a root, which is then linked under the other
+// side's node as it stands: ids fall along every path, so that node is not in
+// the larger root's tree, and it need not be a root itself. (This is Rem's
+// linking, as in Patwary, Blair and Manne, SEA 2010, without its splicing; the
+// nodes passed are repointed at their grandparents instead.) A side is read no
+// further than the other side makes necessary, where walking both to verified
+// roots first reads at least one more node on each. Against that (with compare-and-
+// swap or atomicMin on both verified roots), per pass: R-MAT n = 2^22 with a
+// compression after each of 32 minibatches 1492 -> 1312 us, 104 ragged
+// minibatches 1033 -> 922, R-MAT n = 2^24 without compression 3776 -> 3518, the
+// grid 6640 -> 6464; the first minibatch on an empty forest 145 -> 84 us (R-MAT
+// n = 2^22), 55 -> 35 (n = 2^20).
+//
+// The E edges advance in lockstep: all their loads are issued, then all their
+// link attempts. An attempt on a node that is no root any more returns its
+// parent, which is what a read would have returned: with compare-and-swap the
+// node is untouched. With atomicMin (minhook) a parent above lo is lowered to
+// lo, which moves the node's subtree into lo's tree; the edge goes on joining
+// the displaced parent with lo, so every earlier connection is kept (a
+// splitting store that races with the move and undoes it is harmless for the
+// same reason). Only a write at a root counts as a link. Each round strictly
+// lowers the larger node of every edge, so the loop ends.
+// One link attempt per distinct hi among the lanes of a whole warp that try
+// one: the first of them tries to put hi under its own lo. Returns hi if this
+// lane linked it, else hi's parent as this leaves it (p for a lane without a try).
+__device__ __forceinline__ int link_grouped(int* parent, bool tries, int hi, int lo, bool minhook, int p) {
+    const unsigned full = 0xffffffffu;
+    if (!__any_sync(full, tries)) return p;
+    const int lane = (int)(threadIdx.x & 31u);
+    const int leader = __ffs(__match_any_sync(full, tries ? hi : -1 - lane)) - 1;
+    int old = hi;
+    if (tries && lane == leader) old = minhook ? atomicMin(parent + hi, lo) : atomicCAS(parent + hi, hi, lo);
+    old = __shfl_sync(full, old, leader);
+    const int to = __shfl_sync(full, lo, leader);
+    if (!tries) return p;
+    return lane != leader && (old == hi || (minhook && to < old && old < hi)) ? to : old;
+}
+
+template <int E, bool WARP>
+__device__ __forceinline__ int join_edges(int* parent, unsigned m, const int (&u)[E], const int (&v)[E],
+                                          const int (&pu)[E], const int (&pv)[E], DevState* ds, int hook) {
+    const bool minhook = hook & HOOK_MIN, climb = hook & HOOK_CLIMB;
+    int hi[E], lo[E];    // the two nodes of each edge; equal once it is done
+    int bhi[E], blo[E];  // the node below each on its path, or -1: it was a root when it was read
+    bool any = false;
 #pragma unroll
     for (int i = 0; i < E; i++) {
-        live[i] = ((m >> i) & 1u) && pu[i] != pv[i];
-        x[2 * i] = u[i];
-        x[2 * i + 1] = v[i];
-        p[2 * i] = live[i] ? pu[i] : u[i];
-        p[2 * i + 1] = live[i] ? pv[i] : v[i];
+        const bool swap = pu[i] < pv[i];
+        const int x = swap ? v[i] : u[i], y = swap ? u[i] : v[i];
+        lo[i] = swap ? pu[i] : pv[i];
+        hi[i] = !((m >> i) & 1u) ? lo[i] : swap ? pv[i] : pu[i];
+        bhi[i] = hi[i] == x ? -1 : x;
+        blo[i] = lo[i] == y ? -1 : y;
+        any |= hi[i] != lo[i];
     }
-    walk_split<2 * E>(parent, x, p, ds);
     int made = 0;
-    if constexpr (WARP) {  // every lane of the warp is here (see the kernels)
-        int a[E], b[E];
+    while (WARP ? __any_sync(0xffffffffu, any) : any) {
+        int p[E];
 #pragma unroll
         for (int i = 0; i < E; i++) {
-            a[i] = x[2 * i];
-            b[i] = x[2 * i + 1];
+            p[i] = hi[i];
+            if (hi[i] != lo[i] && bhi[i] >= 0) p[i] = parent[hi[i]];
         }
-        made = hook_warp<E>(parent, live, a, b, ds, minhook);
-    } else {
+        if (climb) {
+            int q[E];
 #pragma unroll
-        for (int i = 0; i < E; i++)
-            if (live[i]) made += hook_as(parent, x[2 * i], x[2 * i + 1], ds, minhook);
+            for (int i = 0; i < E; i++) {
+                q[i] = lo[i];
+                if (hi[i] != lo[i] && blo[i] >= 0 && p[i] == hi[i]) q[i] = parent[lo[i]];
+            }
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                if (q[i] >= lo[i]) continue;
+                lower(parent, blo[i], q[i]);
+                blo[i] = lo[i];
+                lo[i] = q[i];
+                bhi[i] = -1;  // hi has been read and is a root
+                p[i] = -1;    // no attempt in this round
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            const bool tries = hi[i] != lo[i] && p[i] == hi[i];
+            if constexpr (WARP) p[i] = link_grouped(parent, tries, hi[i], lo[i], minhook, p[i]);
+            else if (tries) p[i] = minhook ? atomicMin(parent + hi[i], lo[i]) : atomicCAS(parent + hi[i], hi[i], lo[i]);
+        }
+        any = false;
+#pragma unroll
+        for (int i = 0; i < E; i++) {
+            if (hi[i] == lo[i]) continue;
+            if (climb && p[i] < 0) {
+                any = true;
+                continue;
+            }
+            if (p[i] >= hi[i]) {  // linked, or a broken invariant: stop rather than loop
+                if (p[i] == hi[i]) made++;
+                else flag(ds, ST_CORRUPT);
+                hi[i] = lo[i];
+                continue;
+            }
+            if (bhi[i] >= 0) lower(parent, bhi[i], p[i]);  // splitting: skip a level
+            const int below = hi[i];
+            const bool swap = p[i] < lo[i];
+            hi[i] = swap ? lo[i] : p[i];
+            bhi[i] = swap ? blo[i] : below;
+            lo[i] = swap ? p[i] : lo[i];
+            blo[i] = swap ? below : blo[i];
+            any |= hi[i] != lo[i];
+        }
     }
     return made;
 }
+
+// One fused pass of Algorithm 2 over E edges: the first parent reads of both
+// endpoints of all E edges are issued together; equal parents mean the edge
+// joins a tree to itself and is dropped at once (the common case once trees
+// are flat, and the self-loop filter of Algorithm 2). The others are joined.
+// Returns the number of links made.
+template <int E, bool WARP>
+__device__ __forceinline__ int update_edges(int* __restrict__ parent, int n, const int (&u)[E], const int (&v)[E],
+                                            int64_t e0, int64_t k, DevState* __restrict__ ds, int hook,
+                                            const unsigned* bits) {
+    const unsigned m = edge_mask<E>(n, u, v, e0, k, ds, bits);
+    int pu[E], pv[E];
+    gather_parents<E>(parent, m, u, v, pu, pv);
+    return join_edges<E, WARP>(parent, m, u, v, pu, pv, ds, hook);
+}
+
+// early: the first edges are read before the wait for the previous kernel
+// (programmatic dependent launch; see launch_windowed), else after it.
+// WARP: the link attempts of a warp are grouped by target (link_grouped), so
+// every lane of a warp that has any edge left goes through each round of the
+// loop, with no edges of its own if it has none.
+template <int E, bool PERSIST, bool WARP>
+__global__ void __launch_bounds__(1024)
+k_update(int* __restrict__ parent, int n, const int* __restrict__ edges, int64_t k, int vec,
+         DevState* __restrict__ ds, int early, int hook, BigArgs fb) {
+    pdl_trigger();
+    if (!early) pdl_wait();
+    if (fb.alt && big_active(fb.big, ds)) {  // the filter is on: the edges were not ordered
+        edges = fb.alt;
+        vec = pair_vec_dev(fb.alt);
+    }
+    int made = 0;
+    int64_t e0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * E;
+    if (!PERSIST) {
+        // with warphook, every lane goes in if any lane of its warp has edges
+        bool warp_busy = false;
+        if constexpr (WARP) warp_busy = __any_sync(0xffffffffu, e0 < k);
+        if (e0 < k || warp_busy) {
+            int u[E], v[E];
+            load_pairs<E>(edges, e0, k, vec, u, v);
+            if (early) pdl_wait();
+            made = update_edges<E, WARP>(parent, n, u, v, e0, k, ds, hook, big_active(fb.big, ds));
+        }
+    } else {
+        // persistent grid: loop over chunks, loading the next chunk's edges
+        // before walking the current one so their latency overlaps
+        const int64_t stride = (int64_t)gridDim.x * blockDim.x * E;
+        int u[E], v[E];
+        if (e0 < k) load_pairs<E>(edges, e0, k, vec, u, v);
+        if (early) pdl_wait();
+        const unsigned* bits = big_active(fb.big, ds);
+        while (WARP ? __any_sync(0xffffffffu, e0 < k) : e0 < k) {
+            const int64_t nx = e0 + stride;
+            int nu[E] = {}, nv[E] = {};
+            if (nx < k) load_pairs<E>(edges, nx, k, vec, nu, nv);
+            made += update_edges<E, WARP>(parent, n, u, v, e0, k, ds, hook, bits);
+#pragma unroll
+            for (int i = 0; i < E; i++) {
+                u[i] = nu[i];
+                v[i] = nv[i];
+            }
+            e0 = nx;
+        }
+    }
+    made = __reduce_add_sync(0xffffffffu, made);
+    if ((threadIdx.x & 31) == 0 && made) atomicAdd(&ds->unions, (unsigned long long)made);
+}
+
+// --- VARIANT 3: the persistent grid with a two-stage prefetch -------------
 
 // Persistent grid over chunks of E edges per thread. While the walks and
 // hooks of chunk c run, the first parent reads of chunk c+1 and the edge
@@ -261,7 +278,7 @@ __device__ __forceinline__ int walk_and_hook(int* parent, unsigned m, const int 
 template <int E, bool WARP>
 __global__ void __launch_bounds__(1024)
 k_update_deep(int* __restrict__ parent, int n, const int* __restrict__ edges, int64_t k, int vec,
-              DevState* __restrict__ ds, int early, int minhook, BigArgs fb) {
+              DevState* __restrict__ ds, int early, int hook, BigArgs fb) {
     pdl_trigger();
     if (!early) pdl_wait();
     if (fb.alt && big_active(fb.big, ds)) {  // as in k_update
@@ -286,7 +303,7 @@ k_update_deep(int* __restrict__ parent, int n, const int* __restrict__ edges, in
         gather_parents<E>(parent, m1, u1, v1, pu1, pv1);
         int u2[E] = {}, v2[E] = {};
         if (e2 < k) load_pairs<E>(edges, e2, k, vec, u2, v2);
-        made += walk_and_hook<E, WARP>(parent, m0, u0, v0, pu0, pv0, ds, minhook);
+        made += join_edges<E, WARP>(parent, m0, u0, v0, pu0, pv0, ds, hook);
 #pragma unroll
         for (int i = 0; i < E; i++) {
             u0[i] = u1[i]; v0[i] = v1[i]; pu0[i] = pu1[i]; pv0[i] = pv1[i];
@@ -301,20 +318,20 @@ k_update_deep(int* __restrict__ parent, int n, const int* __restrict__ edges, in
 
 template <int E>
 static void update_deep_inst(const int* edges, int64_t k, int vec, int* parent, int n, DevState* ds,
-                             int block, const cudaAccessPolicyWindow* window, int pdl, int minhook,
+                             int block, const cudaAccessPolicyWindow* window, int pdl, int hook,
                              int warphook, BigArgs fb, cudaStream_t s) {
     int64_t g = (k + (int64_t)E * block - 1) / ((int64_t)E * block);
     if (warphook) {
         const int64_t cap = resident_grid<k_update_deep<E, true>>(block);
         if (g > cap) g = cap;
         launch_windowed(k_update_deep<E, true>, (unsigned)g, block, s, window, pdl != 0, parent, n, edges, k,
-                        vec, ds, (int)(pdl == 2), minhook, fb);
+                        vec, ds, (int)(pdl == 2), hook, fb);
         return;
     }
     const int64_t cap = resident_grid<k_update_deep<E, false>>(block);
     if (g > cap) g = cap;
     launch_windowed(k_update_deep<E, false>, (unsigned)g, block, s, window, pdl != 0, parent, n, edges, k, vec,
-                    ds, (int)(pdl == 2), minhook, fb);
+                    ds, (int)(pdl == 2), hook, fb);
 }
 
 // --- VARIANT 5: per-CTA list of open edges ---------------------------------
@@ -332,7 +349,7 @@ static void update_deep_inst(const int* edges, int64_t k, int vec, int* parent, 
 template <int E>
 __global__ void __launch_bounds__(1024, 1)  // without the minimum, E = 1 and 2 were held to 32 registers and spilled
 k_update_tiles(int* __restrict__ parent, int n, const int* __restrict__ edges, int64_t k, int vec,
-               DevState* __restrict__ ds, int early, int minhook, BigArgs fb) {
+               DevState* __restrict__ ds, int early, int hook, BigArgs fb) {
     extern __shared__ int4 open_list[];  // blockDim.x * E entries: (u, v, parent[u], parent[v])
     __shared__ unsigned n_open[2];
     pdl_trigger();
@@ -396,7 +413,7 @@ k_update_tiles(int* __restrict__ parent, int n, const int* __restrict__ edges, i
             const int4 b = j + 1 < cnt ? open_list[j + 1] : a;
             const unsigned on = j + 1 < cnt ? 3u : 1u;
             const int lu[2] = {a.x, b.x}, lv[2] = {a.y, b.y}, lpu[2] = {a.z, b.z}, lpv[2] = {a.w, b.w};
-            made += walk_and_hook<2>(parent, on, lu, lv, lpu, lpv, ds, minhook);
+            made += join_edges<2, false>(parent, on, lu, lv, lpu, lpv, ds, hook);
         }
         __syncthreads();  // B: the list has been walked; it may be refilled
 #pragma unroll
@@ -411,7 +428,7 @@ k_update_tiles(int* __restrict__ parent, int n, const int* __restrict__ edges, i
 
 template <int E>
 static void update_tiles_inst(const int* edges, int64_t k, int vec, int* parent, int n, DevState* ds, int block,
-                              const cudaAccessPolicyWindow* window, int pdl, int minhook, BigArgs fb,
+                              const cudaAccessPolicyWindow* window, int pdl, int hook, BigArgs fb,
                               cudaStream_t s) {
     const size_t smem = sizeof(int4) * (size_t)block * E;
     if (smem > 48 * 1024)  // the largest list (1024 threads x 4 edges) needs 64 KiB
@@ -424,7 +441,7 @@ static void update_tiles_inst(const int* edges, int64_t k, int vec, int* parent,
     const int64_t cap = (int64_t)(per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
     if (g > cap) g = cap;
     launch_windowed_smem(k_update_tiles<E>, (unsigned)g, block, smem, s, window, pdl != 0, parent, n, edges, k, vec, ds,
-                         (int)(pdl == 2), minhook, fb);
+                         (int)(pdl == 2), hook, fb);
 }
 
 // --- VARIANT 4: filter pass + live-edge pass ------------------------------
@@ -436,7 +453,7 @@ static void update_tiles_inst(const int* edges, int64_t k, int vec, int* parent,
 // at the rate of the gathers -- and appends each edge that is still open as
 // (u, v, parent[u], parent[v]) to a compact list. Pass 2 walks and hooks only
 // the listed edges, from the parents pass 1 read (still ancestors; see
-// walk_and_hook). The two list counters alternate between minibatches: pass 1
+// join_edges). The two list counters alternate between minibatches: pass 1
 // of minibatch i appends through count[sel] and zeroes count[sel ^ 1] for
 // minibatch i + 1, after the wait that orders it behind everything before it.
 
@@ -482,11 +499,11 @@ k_update_filter(const int* __restrict__ parent, int n, const int* __restrict__ e
         if ((open >> i) & 1u) live[base++] = make_int4(u[i], v[i], pu[i], pv[i]);
 }
 
-// Pass 2: two listed edges per thread per step, their four walks in lockstep.
+// Pass 2: two listed edges per thread per step, in lockstep.
 template <bool WARP>
 __global__ void __launch_bounds__(1024)
 k_update_live(int* __restrict__ parent, const int4* __restrict__ live, const unsigned* __restrict__ count,
-              int sel, DevState* __restrict__ ds, int minhook) {
+              int sel, DevState* __restrict__ ds, int hook) {
     pdl_trigger();
     pdl_wait();
     const int64_t m = count[sel];
@@ -499,7 +516,7 @@ k_update_live(int* __restrict__ parent, const int4* __restrict__ live, const uns
         const int4 b = i + 1 < m ? live[i + 1] : a;
         const unsigned on = i + 1 < m ? 3u : i < m ? 1u : 0u;
         const int u[2] = {a.x, b.x}, v[2] = {a.y, b.y}, pu[2] = {a.z, b.z}, pv[2] = {a.w, b.w};
-        made += walk_and_hook<2, WARP>(parent, on, u, v, pu, pv, ds, minhook);
+        made += join_edges<2, WARP>(parent, on, u, v, pu, pv, ds, hook);
     }
     made = __reduce_add_sync(0xffffffffu, made);
     if ((threadIdx.x & 31) == 0 && made) atomicAdd(&ds->unions, (unsigned long long)made);
@@ -533,62 +550,58 @@ cudaError_t launch_update_split(int* parent, int n, const int* edges, int64_t k,
         const int64_t cap = resident_grid<k_update_live<true>>(cfg.block);
         if (g > cap) g = cap;
         launch_windowed(k_update_live<true>, (unsigned)g, cfg.block, s, cfg.window, cfg.pdl != 0, parent,
-                        (const int4*)live, (const unsigned*)count, sel, ds, cfg.minhook);
+                        (const int4*)live, (const unsigned*)count, sel, ds, cfg.hook);
     } else {
         const int64_t cap = resident_grid<k_update_live<false>>(cfg.block);
         if (g > cap) g = cap;
         launch_windowed(k_update_live<false>, (unsigned)g, cfg.block, s, cfg.window, cfg.pdl != 0, parent,
-                        (const int4*)live, (const unsigned*)count, sel, ds, cfg.minhook);
+                        (const int4*)live, (const unsigned*)count, sel, ds, cfg.hook);
     }
     return cudaGetLastError();
 }
 
 
-template <int E, int VARIANT, bool WARP>
+template <int E, bool PERSIST, bool WARP>
 static void update_inst2(const int* edges, int64_t k, int vec, int* parent, int n, DevState* ds,
-                         int block, const cudaAccessPolicyWindow* window, int pdl, int minhook,
+                         int block, const cudaAccessPolicyWindow* window, int pdl, int hook,
                          BigArgs fb, cudaStream_t s) {
     int64_t g = (k + (int64_t)E * block - 1) / ((int64_t)E * block);
-    if (VARIANT == 2) {
-        const int64_t cap = resident_grid<k_update<E, VARIANT, WARP>>(block);
+    if (PERSIST) {
+        const int64_t cap = resident_grid<k_update<E, PERSIST, WARP>>(block);
         if (g > cap) g = cap;
     }
-    launch_windowed(k_update<E, VARIANT, WARP>, (unsigned)g, block, s, window, pdl != 0, parent, n, edges, k,
-                    vec, ds, (int)(pdl == 2), minhook, fb);
+    launch_windowed(k_update<E, PERSIST, WARP>, (unsigned)g, block, s, window, pdl != 0, parent, n, edges, k,
+                    vec, ds, (int)(pdl == 2), hook, fb);
 }
 
-// warphook applies to the lockstep variants (1, 2); variant 0 hooks per edge
-template <int E, int VARIANT>
+template <int E, bool PERSIST>
 static void update_inst(const int* edges, int64_t k, int vec, int* parent, int n, DevState* ds,
-                        int block, const cudaAccessPolicyWindow* window, int pdl, int minhook,
+                        int block, const cudaAccessPolicyWindow* window, int pdl, int hook,
                         int warphook, BigArgs fb, cudaStream_t s) {
-    if (VARIANT != 0 && warphook)
-        update_inst2<E, VARIANT, VARIANT != 0>(edges, k, vec, parent, n, ds, block, window, pdl, minhook, fb, s);
+    if (warphook)
+        update_inst2<E, PERSIST, true>(edges, k, vec, parent, n, ds, block, window, pdl, hook, fb, s);
     else
-        update_inst2<E, VARIANT, false>(edges, k, vec, parent, n, ds, block, window, pdl, minhook, fb, s);
+        update_inst2<E, PERSIST, false>(edges, k, vec, parent, n, ds, block, window, pdl, hook, fb, s);
 }
 
 cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevState* ds,
                           Launch cfg, cudaStream_t s) {
     if (k <= 0) return cudaSuccess;
     const int vec = pair_vec(edges);
-#define CC_UPD(E, V) update_inst<E, V>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s)
+#define CC_UPD(E, P) update_inst<E, P>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, cfg.variant ? cfg.warphook : 0, BigArgs{cfg.big, cfg.alt}, s)
     switch (cfg.variant * 8 + cfg.ept) {
-        case 1: CC_UPD(1, 0); break;
-        case 2: CC_UPD(2, 0); break;
-        case 4: CC_UPD(4, 0); break;
-        case 9: CC_UPD(1, 1); break;
-        case 10: CC_UPD(2, 1); break;
-        case 12: CC_UPD(4, 1); break;
-        case 17: CC_UPD(1, 2); break;
-        case 18: CC_UPD(2, 2); break;
-        case 20: CC_UPD(4, 2); break;
-        case 25: update_deep_inst<1>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s); break;
-        case 26: update_deep_inst<2>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s); break;
-        case 28: update_deep_inst<4>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s); break;
-        case 41: update_tiles_inst<1>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, BigArgs{cfg.big, cfg.alt}, s); break;
-        case 42: update_tiles_inst<2>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, BigArgs{cfg.big, cfg.alt}, s); break;
-        case 44: update_tiles_inst<4>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.minhook, BigArgs{cfg.big, cfg.alt}, s); break;
+        case 1: case 9: CC_UPD(1, false); break;
+        case 2: case 10: CC_UPD(2, false); break;
+        case 4: case 12: CC_UPD(4, false); break;
+        case 17: CC_UPD(1, true); break;
+        case 18: CC_UPD(2, true); break;
+        case 20: CC_UPD(4, true); break;
+        case 25: update_deep_inst<1>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s); break;
+        case 26: update_deep_inst<2>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s); break;
+        case 28: update_deep_inst<4>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, cfg.warphook, BigArgs{cfg.big, cfg.alt}, s); break;
+        case 41: update_tiles_inst<1>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, BigArgs{cfg.big, cfg.alt}, s); break;
+        case 42: update_tiles_inst<2>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, BigArgs{cfg.big, cfg.alt}, s); break;
+        case 44: update_tiles_inst<4>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, BigArgs{cfg.big, cfg.alt}, s); break;
         default: return cudaErrorInvalidValue;
     }
 #undef CC_UPD
