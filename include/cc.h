@@ -77,8 +77,9 @@ typedef enum {
                                     over is repointed at its grandparent, which shortens paths for
                                     later operations */
     CC_OPT_PROFILE = 5,          /* 1: time every kernel with CUDA events on the handle's stream */
-    CC_OPT_UPDATE_VARIANT = 6,   /* Bulk-Update kernel: 0 and 1 one chunk of edges per thread, 2 = 1
-                                    on a persistent grid that prefetches the next edges, 3 = 2 that also has the next chunk's first
+    CC_OPT_UPDATE_VARIANT = 6,   /* Bulk-Update kernel: 0 = 1 for minibatches below 2^18 edges, 5 in
+                                    CTAs of 128 threads from there; 1 = one chunk of edges per
+                                    thread; 2 = 1 on a persistent grid that prefetches the next edges, 3 = 2 that also has the next chunk's first
                                     parent reads in flight during this chunk's walks, 4 = two
                                     kernels: a filter pass that reads every edge's first parents
                                     and lists the edges whose parents differ (16 B each; the list,

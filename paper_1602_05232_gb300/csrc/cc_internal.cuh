@@ -38,7 +38,7 @@ enum : int {
 struct Launch {
     int block;        // threads per block, multiple of 32
     int ept;          // edges (pairs) per thread: 1, 2 or 4
-    int variant = 0;  // update kernel: 0 and 1 one chunk per thread, 2 persistent + prefetch,
+    int variant = 0;  // update kernel: 0 = 1 or 5 by size, 1 one chunk per thread, 2 persistent + prefetch,
                       // 3 persistent + two-stage prefetch (edges two chunks ahead, parents one),
                       // 4 filter pass + live-edge pass (launch_update_split),
                       // 5 persistent tiles whose open edges the whole CTA walks from a shared-memory list
@@ -69,11 +69,12 @@ struct BigArgs {
     const int* alt = nullptr;
 };
 
-// A persistent grid for KERNEL at `block` threads (no dynamic shared memory):
-// resident CTAs per SM x SMs of the current device. Cached per host thread,
-// device and block size, so neither threads nor different GPUs share an entry.
+// A persistent grid for KERNEL at `block` threads and `smem` bytes of dynamic
+// shared memory (the same for every call with that block): resident CTAs per
+// SM x SMs of the current device. Cached per host thread, device and block
+// size, so neither threads nor different GPUs share an entry.
 template <auto KERNEL>
-static int resident_grid(int block) {
+static int resident_grid(int block, size_t smem = 0) {
     thread_local int cache[16][33] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -81,7 +82,7 @@ static int resident_grid(int block) {
     if (slot && *slot) return *slot;
     int per_sm = 0, sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, block, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KERNEL, block, smem);
     const int c = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
     if (slot) *slot = c;
     return c;

@@ -433,12 +433,8 @@ static void update_tiles_inst(const int* edges, int64_t k, int vec, int* parent,
     const size_t smem = sizeof(int4) * (size_t)block * E;
     if (smem > 48 * 1024)  // the largest list (1024 threads x 4 edges) needs 64 KiB
         cudaFuncSetAttribute(k_update_tiles<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm = 0, sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_update_tiles<E>, block, smem);
     int64_t g = (k + (int64_t)E * block - 1) / ((int64_t)E * block);
-    const int64_t cap = (int64_t)(per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+    const int64_t cap = resident_grid<k_update_tiles<E>>(block, smem);
     if (g > cap) g = cap;
     launch_windowed_smem(k_update_tiles<E>, (unsigned)g, block, smem, s, window, pdl != 0, parent, n, edges, k, vec, ds,
                          (int)(pdl == 2), hook, fb);
@@ -584,10 +580,24 @@ static void update_inst(const int* edges, int64_t k, int vec, int* parent, int n
         update_inst2<E, PERSIST, false>(edges, k, vec, parent, n, ds, block, window, pdl, hook, fb, s);
 }
 
+// Variant 0 takes the tile kernel (variant 5) in CTAs of 128 threads from this
+// many edges, about one wave of its tiles, and one chunk per thread below.
+// Whole passes with a compression after each minibatch, 2 edges per thread, one
+// chunk per thread (256 threads) against tiles (128): R-MAT n = 2^22 with 2^20
+// edges a minibatch 1277 and 926 us, 2^18 583 and 540, 2^17 470 and 518; a 3001 x
+// 3001 mesh 1225 and 888 with 2^20, 1042 and 992 with 2^18; R-MAT n = 2^24 with
+// 2^22 2230 and 1315; 50,000 edges on 10^6 vertices 931 and 1098. Tiles of 256
+// threads: 995 us with 2^20, 535 with 2^18.
+constexpr int64_t kTileEdges = 1 << 18;
+
 cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevState* ds,
                           Launch cfg, cudaStream_t s) {
     if (k <= 0) return cudaSuccess;
     const int vec = pair_vec(edges);
+    if (cfg.variant == 0 && k >= kTileEdges) {
+        cfg.variant = 5;
+        cfg.block = 128;
+    }
 #define CC_UPD(E, P) update_inst<E, P>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, cfg.variant ? cfg.warphook : 0, BigArgs{cfg.big, cfg.alt}, s)
     switch (cfg.variant * 8 + cfg.ept) {
         case 1: case 9: CC_UPD(1, false); break;

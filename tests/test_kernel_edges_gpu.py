@@ -172,3 +172,32 @@ def test_query_walks_answer_as_the_roots_do(cc, k, shape):
             assert got[-1] == 0 and np.array_equal(got[:-1], want[:-1])
             with pytest.raises(cc.CCError):
                 f.sync()
+
+
+# ---------------------------------------------------------------- Bulk-Update
+
+@pytest.mark.parametrize("ept", [1, 2, 4])
+@pytest.mark.parametrize("k", [1, (1 << 18) - 1, 1 << 18, (1 << 18) + 127])
+def test_update_on_both_sides_of_the_tile_rule(cc, k, ept):
+    """Whole minibatches on a sparse, a dense and an already joined forest."""
+    import oracle
+    r = np.random.default_rng(k + ept)
+    for n in (1000, 150_001, 2_000_003):
+        ref = oracle.OracleUF(n)
+        f = cc.Forest(n, edges_per_thread=ept)
+        g = cc.Forest(n, edges_per_thread=ept, compress_every=0, hook=1)
+        for step in range(3):
+            e = r.integers(0, n, size=(k, 2)).astype(np.int32)
+            e[::5] = np.sort(e[::5], axis=1)
+            e[1::9, 0] = n // 2                     # a hub
+            ref.bulk_update(e)
+            for x in (f, g):
+                x.bulk_update(dev(e, shift=step % 2))
+                assert x.components() == ref.components
+        for x in (f, g):
+            assert np.array_equal(x.labels().cpu().numpy(), ref.labels())
+            x.sync()
+            bad = np.array([[0, n], [-1, 0], [0, 1]], dtype=np.int32).repeat(max(1, k // 3), axis=0)
+            x.bulk_update(dev(bad))
+            with pytest.raises(cc.CCError):
+                x.sync()
