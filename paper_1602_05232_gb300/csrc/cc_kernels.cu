@@ -992,7 +992,11 @@ cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_
 // root of v is ds->big_root), one 32-bit word per 8 lanes (a warp covers 128
 // consecutive vertices); every lane of a warp takes part, so threads past n
 // do not leave early. (Counting the marked vertices here, one atomic per warp
-// on one word, doubled the pass: launch_big_count does it on demand.)
+// on one word, doubled the pass: launch_big_count does it on demand.) With BIG
+// four parents are written back as one vector if any changed: these passes come
+// after several minibatches, so that most have (2^26 vertices of the grid: 178 ->
+// 158 us a pass); where one minibatch went before, single stores are the faster
+// ones (2^25 vertices of an R-MAT graph: 45 and 48 us).
 // As a dependent launch it starts while the update drains, where a plain launch
 // costs a boundary of about 2 us on each side (ragged minibatches on 10^6
 // vertices, three kernels a step: 1250 -> 1011 us for 104 steps). It has no
@@ -1016,7 +1020,7 @@ k_compress_all(int* __restrict__ parent, int64_t n, int* __restrict__ out,
     }
 #pragma unroll
     for (int i = 0; i < 4; i++) {
-        x[i] = v0 + i < n ? (int)(v0 + i) : 0;  // past n: a walk of length 0
+        x[i] = (BIG && full) || v0 + i < n ? (int)(v0 + i) : 0;  // past n: a walk of length 0
         p[i] = p0[i];
     }
     while (true) {
@@ -1031,11 +1035,14 @@ k_compress_all(int* __restrict__ parent, int64_t n, int* __restrict__ out,
         }
         if (!any) break;
     }
+    bool changed = false;
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         if (p[i] > x[i]) flag(ds, ST_CORRUPT);
-        if (v0 + i < n && x[i] != p0[i]) parent[v0 + i] = x[i];
+        if ((!BIG || !full) && v0 + i < n && x[i] != p0[i]) parent[v0 + i] = x[i];
+        changed |= x[i] != p0[i];
     }
+    if (BIG && full && changed) reinterpret_cast<int4*>(parent)[v0 / 4] = make_int4(x[0], x[1], x[2], x[3]);
     if (OUT) {
         if (full) {
             reinterpret_cast<int4*>(out)[v0 / 4] = make_int4(x[0], x[1], x[2], x[3]);
@@ -1051,7 +1058,7 @@ k_compress_all(int* __restrict__ parent, int64_t n, int* __restrict__ out,
         unsigned nib = 0;
 #pragma unroll
         for (int i = 0; i < 4; i++)
-            if (v0 + i < n && x[i] == R) nib |= 1u << i;
+            if ((full || v0 + i < n) && x[i] == R) nib |= 1u << i;
         const unsigned lane = threadIdx.x & 31u;
         unsigned w = nib << ((lane & 7u) * 4u);
         w |= __shfl_xor_sync(0xffffffffu, w, 1);
