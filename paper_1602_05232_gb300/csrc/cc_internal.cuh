@@ -146,6 +146,16 @@ cudaError_t launch_reset(int* parent, int64_t n, DevState* ds, int block, bool p
 cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevState* ds,
                           Launch cfg, cudaStream_t s);
 
+// A Bulk-Update that one CTA does in shared memory, leaving every vertex pointed
+// at its root. Against the general update and its compression pass, whole steps
+// with a query each, the host enqueueing: 8.1-8.9 -> 6.0-6.9 us for up to 4096
+// edges on up to 4096 vertices and 1024 on 8192, 8.5 -> 8.1 for 4096 on 8192,
+// but 8.5 -> 10.3 for 8192 on 8192 and 8.7 -> 10.9 for 8192 on 4096.
+constexpr int64_t kSmallVertices = 8192, kSmallEdges = 4096;
+bool small_update(int64_t n, int64_t k);
+cudaError_t launch_update_small(int* parent, int n, const int* edges, int64_t k, DevState* ds, int pdl,
+                                cudaStream_t s);
+
 // Bulk-Update as two kernels (update variant 4): a filter pass that reads the
 // first parents of every edge and lists the edges whose parents differ as
 // (u, v, parent[u], parent[v]) in live[] (room for k entries), then a pass

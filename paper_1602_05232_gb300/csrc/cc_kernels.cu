@@ -580,6 +580,104 @@ static void update_inst(const int* edges, int64_t k, int vec, int* parent, int n
         update_inst2<E, PERSIST, false>(edges, k, vec, parent, n, ds, block, window, pdl, hook, fb, s);
 }
 
+// A small minibatch on a small forest in one CTA, with the forest in shared
+// memory: loaded, joined as in join_edges, flattened and written back, so that
+// no compression is left to do. Bound by latency: the chains of dependent
+// reads and links that many edges on few vertices make (most of all on an empty
+// forest) take tens of cycles a step here instead of hundreds of nanoseconds a
+// step in L2, and one launch takes the place of two: four minibatches of 4096
+// edges on an empty forest of 4096 vertices, each with a query, 37.4 -> 34.3 us.
+constexpr int kSmallBlock = 1024;
+
+__global__ void __launch_bounds__(kSmallBlock)
+k_update_small(int* __restrict__ parent, int n, const int* __restrict__ edges, int k, int vec,
+               DevState* __restrict__ ds, int early) {
+    extern __shared__ int4 small_forest[];
+    int* sp = reinterpret_cast<int*>(small_forest);
+    __shared__ int part[kSmallBlock / 32];
+    pdl_trigger();
+    const int tid = threadIdx.x;
+    int u[2] = {}, v[2] = {};
+    if (!early) pdl_wait();
+    if (2 * tid < k) load_pairs<2>(edges, 2 * tid, k, vec, u, v);
+    if (early) pdl_wait();
+    const int quads = n / 4;
+    for (int c = tid; c < quads; c += kSmallBlock) small_forest[c] = reinterpret_cast<const int4*>(parent)[c];
+    if (tid < n - 4 * quads) sp[4 * quads + tid] = parent[4 * quads + tid];
+    __syncthreads();
+    int made = 0;
+    bool bad = false;
+    for (int i0 = 2 * tid; i0 < k; i0 += 2 * kSmallBlock) {
+        int nu[2] = {}, nv[2] = {};
+        if (i0 + 2 * kSmallBlock < k) load_pairs<2>(edges, i0 + 2 * kSmallBlock, k, vec, nu, nv);
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            if (i0 + i >= k) continue;
+            if (!(in_range(u[i], n) && in_range(v[i], n))) {
+                bad = true;
+                continue;
+            }
+            int hi = u[i] > v[i] ? u[i] : v[i], lo = u[i] > v[i] ? v[i] : u[i], bhi = -1, blo = -1;
+            while (hi != lo) {
+                volatile int* vp = sp;
+                int p = vp[hi];
+                if (p == hi) {
+                    p = atomicCAS(sp + hi, hi, lo);
+                    if (p == hi) {
+                        made++;
+                        break;
+                    }
+                }
+                if (p > hi) {  // broken invariant: stop rather than loop
+                    flag(ds, ST_CORRUPT);
+                    break;
+                }
+                if (bhi >= 0) vp[bhi] = p;  // splitting: skip a level
+                const int below = hi;
+                const bool swap = p < lo;
+                hi = swap ? lo : p;
+                bhi = swap ? blo : below;
+                lo = swap ? p : lo;
+                blo = swap ? below : blo;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            u[i] = nu[i];
+            v[i] = nv[i];
+        }
+    }
+    if (bad) flag(ds, ST_RANGE);
+    made = __reduce_add_sync(0xffffffffu, made);
+    if ((tid & 31) == 0) part[tid >> 5] = made;
+    __syncthreads();
+    if (tid == 0) {
+        int t = 0;
+        for (int w = 0; w < kSmallBlock / 32; w++) t += part[w];
+        if (t) atomicAdd(&ds->unions, (unsigned long long)t);
+    }
+    for (int c = tid; c < quads; c += kSmallBlock) {
+        const int4 q = small_forest[c];
+        const int4 w = make_int4(walk_root(sp, q.x, sp[q.x]), walk_root(sp, q.y, sp[q.y]),
+                                 walk_root(sp, q.z, sp[q.z]), walk_root(sp, q.w, sp[q.w]));
+        reinterpret_cast<int4*>(parent)[c] = w;
+    }
+    if (tid < n - 4 * quads) {
+        const int x = sp[4 * quads + tid];
+        parent[4 * quads + tid] = walk_root(sp, x, sp[x]);
+    }
+}
+
+bool small_update(int64_t n, int64_t k) { return n <= kSmallVertices && k <= kSmallEdges; }
+
+cudaError_t launch_update_small(int* parent, int n, const int* edges, int64_t k, DevState* ds, int pdl,
+                                cudaStream_t s) {
+    if (k <= 0) return cudaSuccess;
+    launch_windowed_smem(k_update_small, 1u, kSmallBlock, sizeof(int4) * (size_t)((n + 3) / 4), s, nullptr, pdl != 0,
+                         parent, n, edges, (int)k, pair_vec(edges), ds, (int)(pdl == 2));
+    return cudaGetLastError();
+}
+
 // Variant 0 takes the tile kernel (variant 5) in CTAs of 128 threads from this
 // many edges, about one wave of its tiles, and one chunk per thread below.
 // Whole passes with a compression after each minibatch, 2 edges per thread, one

@@ -201,3 +201,43 @@ def test_update_on_both_sides_of_the_tile_rule(cc, k, ept):
             x.bulk_update(dev(bad))
             with pytest.raises(cc.CCError):
                 x.sync()
+
+
+@pytest.mark.parametrize("n", [1, 2, 5, 1023, 4096, 8191, 8192, 8193])
+@pytest.mark.parametrize("k", [1, 2, 2047, 2049, 4096, 4097])
+def test_small_update_equals_the_general_one(cc, n, k):
+    """Both sides of the size rule, on an empty forest, on a deep one that was
+    loaded and between larger minibatches, for every compression policy."""
+    import oracle
+    r = np.random.default_rng(n * 5000 + k)
+    par = np.maximum(np.arange(n) - 1 - r.integers(0, 3, n), 0).astype(np.int32)
+    par = np.where(r.random(n) < 0.3, np.arange(n), par).astype(np.int32)
+    batches = [r.integers(0, n, size=(x, 2)).astype(np.int32) for x in (k, k, 6000, k)]
+    batches[1][: k // 2] = batches[0][: k // 2]
+    for opts in ({}, {"compress_every": 0}, {"compress_every": 2, "hook": 1}, {"compress_scope": 1}, {"pdl": 2}):
+        f, g = cc.Forest(n, **opts), cc.Forest(n, **{**opts, "update_variant": 1})
+        for start in ("empty", "loaded"):
+            ref = oracle.OracleUF(n)
+            if start == "loaded":
+                for x in (f, g):
+                    x.reset()
+                    x.load_forest(dev(par))
+                ref.bulk_update(np.stack([np.arange(n, dtype=np.int32), par], axis=1))
+            for i, e in enumerate(batches):
+                ref.bulk_update(e)
+                q = dev(r.integers(0, n, size=(777, 2)).astype(np.int32))
+                for x in (f, g):
+                    x.bulk_update(dev(e, shift=i % 2))
+                    assert x.components() == ref.components, (opts, start, i)
+                    assert np.array_equal(x.bulk_query(q).cpu().numpy(), ref.bulk_query(q.cpu().numpy()))
+            for x in (f, g):
+                assert np.array_equal(x.labels().cpu().numpy(), ref.labels())
+                x.sync()
+    bad = np.array([[0, 0], [n, 0], [0, -1]], dtype=np.int32)[np.arange(min(k, 3))]
+    f = cc.Forest(n)
+    f.bulk_update(dev(bad))
+    assert f.components() == n
+    if len(bad) > 1:
+        with pytest.raises(cc.CCError) as ex:
+            f.sync()
+        assert ex.value.status == cc.CC_ERR_RANGE
