@@ -128,7 +128,16 @@ def device_can_read(t: torch.Tensor) -> bool:
     return bool(ok.value)
 
 
+_Tensor, _I32, _U8 = torch.Tensor, torch.int32, torch.uint8
+
+
 def _pairs_ptr(t: torch.Tensor, name: str) -> tuple[int, int]:
+    # What nearly every call passes, with as few calls into torch as it takes:
+    # on small minibatches the enqueueing host is what bounds a step.
+    if type(t) is _Tensor and t.is_cuda and t.dtype is _I32 and t.is_contiguous():
+        m = t.numel()
+        if not m & 1:
+            return t.data_ptr(), m >> 1
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name}: expected a tensor")
     if not t.is_cuda and not (t.is_pinned() and device_can_read(t)):
@@ -164,6 +173,7 @@ class Forest:
                   self._L)
             self.offsets = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
         self._h = h
+        self._bulk_update, self._bulk_query = self._L.cc_bulk_update, self._L.cc_bulk_query
         self.n = int(self.offsets[-1])
         self.set_stream(stream)
         for k, v in options.items():
@@ -207,10 +217,18 @@ class Forest:
     # bulk operations ---------------------------------------------------
     def bulk_update(self, edges: torch.Tensor) -> None:
         p, k = _pairs_ptr(edges, "edges")
-        check(self._L.cc_bulk_update(self._h, p, k), self._L)
+        status = self._bulk_update(self._h, p, k)
+        if status:
+            check(status, self._L)
 
     def bulk_query(self, pairs: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         p, k = _pairs_ptr(pairs, "pairs")
+        if (type(out) is _Tensor and out.is_cuda and out.dtype is _U8 and out.is_contiguous()
+                and out.numel() >= k):
+            status = self._bulk_query(self._h, p, k, out.data_ptr())
+            if status:
+                check(status, self._L)
+            return out
         if out is None:
             out = (torch.empty(k, dtype=torch.uint8, device=pairs.device) if pairs.is_cuda
                    else torch.empty(k, dtype=torch.uint8, pin_memory=True))
