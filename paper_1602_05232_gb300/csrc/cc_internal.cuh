@@ -227,10 +227,11 @@ struct SegLaunch {
     int ept;       // edges (pairs) per thread per step: 1, 2 or 4
     int smem_cap;  // graphs of at most this many vertices run in shared memory (<= 65536)
     int max_ctas;  // cap on the persistent grid (0 = one wave of resident CTAs)
-    int grid = 0;  // set by prepare_segmented
+    int grid = 0;  // set by prepare_segmented, as is
+    int depth = 0; // the chunks of pairs in shared memory per CTA (2 to 4)
 };
 
-// Sets the kernel's shared-memory attribute and the persistent grid size.
+// Sets the kernel's shared-memory attribute, the ring's depth and the persistent grid size.
 // Call before launching or capturing.
 cudaError_t prepare_segmented(SegLaunch& cfg);
 

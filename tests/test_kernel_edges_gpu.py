@@ -241,3 +241,49 @@ def test_small_update_equals_the_general_one(cc, n, k):
         with pytest.raises(cc.CCError) as ex:
             f.sync()
         assert ex.value.status == cc.CC_ERR_RANGE
+
+
+# --------------------------------------------------------------- batched form
+
+@pytest.mark.parametrize("opts", [{}, {"seg_block": 1024, "seg_edges_per_thread": 2},
+                                  {"seg_block": 64, "seg_edges_per_thread": 4},
+                                  {"seg_block": 1024, "seg_edges_per_thread": 4},
+                                  {"seg_block": 256, "seg_smem_cap": 3000}])
+def test_batched_operations_of_all_lengths(cc, opts):
+    """More operations than are staged at once, empty ones, lengths around the
+    chunks of every launch shape, and data at 4, 8 and 16-byte alignment."""
+    import oracle
+    r = np.random.default_rng(7)
+    sizes = [1, 2, 700, 3001, 65536]
+    f = cc.Forest.segmented(sizes, **opts)
+    refs = [oracle.OracleUF(n) for n in sizes]
+    lengths = [0, 1, 2, 3, 63, 64, 65, 255, 256, 257, 1023, 1025, 2047, 2048, 2049, 4095, 4097, 0, 9000]
+    ops, want, outs = [], [], []
+    for step in range(2):
+        for g, n in enumerate(sizes):
+            # 1400 short operations on one graph: more than two stagings
+            for i, k in enumerate([1] * 1400 if g == 2 and step else lengths * (2 if n > 2 else 1)):
+                p = r.integers(0, n, size=(k, 2)).astype(np.int32)
+                d = dev(p, shift=i % 4)
+                if i % 2:
+                    out = torch.full((k + 1,), 7, dtype=torch.uint8, device="cuda")
+                    ops.append((g, cc.OP_QUERY, d, out[i % 3 == 0:][:k]))
+                    want.append(refs[g].bulk_query(p))
+                    outs.append(ops[-1][3])
+                else:
+                    ops.append((g, cc.OP_UPDATE, d, None))
+                    refs[g].bulk_update(p)
+        f.submit(ops if step else ops[:])
+        f.sync()
+        for got, exp in zip(outs, want):
+            assert np.array_equal(got.cpu().numpy(), exp)
+        ops, want, outs = [], [], []
+        lab = f.labels().cpu().numpy()
+        for g, ref in enumerate(refs):
+            a, b = f.offsets[g], f.offsets[g + 1]
+            assert np.array_equal(lab[a:b] - a, ref.labels())
+    bad = [(4, cc.OP_UPDATE, dev([[0, 65536], [3, 4]]), None)]
+    f.submit(bad)
+    with pytest.raises(cc.CCError) as ex:
+        f.sync()
+    assert ex.value.status == cc.CC_ERR_RANGE
