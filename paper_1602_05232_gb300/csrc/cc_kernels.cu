@@ -22,6 +22,8 @@ static inline unsigned blocks_for(int64_t work, int64_t per_block) {
 // as two memsets in front they were two more operations on the stream). Kernels
 // that are launched as dependents may read big_root before their own wait; they
 // start once all CTAs here have exited, the first one after its write is visible.
+// Four vectors per thread: with one, CTAs were launched more slowly than they
+// wrote (2^26 vertices in CTAs of 128 threads: 72 -> 39 us, 6.9 TB/s).
 __global__ void k_reset(int* __restrict__ parent, int64_t n, DevState* __restrict__ ds) {
     pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -29,18 +31,22 @@ __global__ void k_reset(int* __restrict__ parent, int64_t n, DevState* __restric
         ds->big_root = -1;
         __threadfence();
     }
-    int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (v0 + 4 <= n) {
-        int x = (int)v0;
-        reinterpret_cast<int4*>(parent)[v0 / 4] = make_int4(x, x + 1, x + 2, x + 3);
-    } else {
-        for (int64_t v = v0; v < n; v++) parent[v] = (int)v;
+    const int64_t q0 = (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int64_t v0 = (q0 + (int64_t)i * blockDim.x) * 4;
+        if (v0 + 4 <= n) {
+            int x = (int)v0;
+            reinterpret_cast<int4*>(parent)[v0 / 4] = make_int4(x, x + 1, x + 2, x + 3);
+        } else {
+            for (int64_t v = v0; v < n; v++) parent[v] = (int)v;
+        }
     }
 }
 
 cudaError_t launch_reset(int* parent, int64_t n, DevState* ds, int block, bool pdl, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    launch_windowed(k_reset, blocks_for(n, 4LL * block), block, s, nullptr, pdl, parent, n, ds);
+    launch_windowed(k_reset, blocks_for(n, 16LL * block), block, s, nullptr, pdl, parent, n, ds);
     return cudaGetLastError();
 }
 
