@@ -216,12 +216,6 @@ cc::Launch cfg_of(const cc_ctx* c) {
                       (int)c->opt[CC_OPT_HOOK_WARP], c->opt[CC_OPT_BIG_FILTER] > 0 ? c->big : nullptr};
 }
 
-// The largest-component bitmap no longer describes the forest (reset, or a
-// forest loaded from outside): off until the next full compression pass.
-cudaError_t big_invalidate(cc_ctx* c) {
-    return cudaMemsetAsync(&c->ds->big_root, 0xff, sizeof(int), c->stream);
-}
-
 cc_status check_pairs(const int32_t* p, int64_t k, const char* name) {
     if (k < 0 || k > INT32_MAX) return fail(CC_ERR_ARG, "%s: k = %lld out of [0, 2^31-1]", name, (long long)k);
     if (k > 0 && !p) return fail(CC_ERR_ARG, "%s: null array with k > 0", name);
@@ -784,7 +778,10 @@ cc_status cc_labels(cc_ctx* c, int32_t* out) {
         if (s == CC_OK) c->flat = true;
         return s;
     }
+    // flat already: the parents are the labels
+    const bool copy = c->flat && reinterpret_cast<uintptr_t>(out) % 16 == 0;
     cc_status s = run(c, CC_K_LABELS, "labels", [&] {
+        if (copy) return cc::launch_copy_ids(c->parent, c->n, out, c->opt[CC_OPT_PDL] != 0, c->stream);
         return cc::launch_compress_all(c->parent, c->n, out, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream);
     });
     if (s == CC_OK) c->flat = true;
@@ -797,22 +794,18 @@ cc_status cc_load_labels(cc_ctx* c, const int32_t* labels) {
     if (reinterpret_cast<uintptr_t>(labels) % 4 != 0) return fail(CC_ERR_ARG, "cc_load_labels: not 4-byte aligned");
     if (c->G > 1) return fail(CC_ERR_UNSUPPORTED, "cc_load_labels on a segmented handle");
     CC_DEVICE(c);
-    cudaError_t e = cudaMemsetAsync(&c->ds->labels_bad, 0, sizeof(unsigned), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&c->ds->roots, 0, sizeof(unsigned long long), c->stream);
+    cudaError_t e = cudaMemsetAsync(&c->ds->checked, 0, sizeof(cc::DevState::Checked), c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cc_load_labels");
     cc_status s = run(c, CC_K_LOAD, "load_labels(validate)", [&] {
         return cc::launch_validate_labels(labels, c->n, c->ds, c->stream);
     });
     if (s != CC_OK) return s;
-    cc::DevState h;
-    e = cudaMemcpyAsync(&h, c->ds, sizeof h, cudaMemcpyDeviceToHost, c->stream);
+    cc::DevState::Checked h;
+    e = cudaMemcpyAsync(&h, &c->ds->checked, sizeof h, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cc_load_labels: read back");
-    if (h.labels_bad) return fail(CC_ERR_LABELS, "cc_load_labels: not a minimum-id labelling (need 0 <= l[v] <= v, l[l[v]] == l[v])");
-    unsigned long long unions = (unsigned long long)c->n - h.roots;
-    e = cudaMemcpyAsync(c->parent, labels, (size_t)c->n * sizeof(int), cudaMemcpyDeviceToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&c->ds->unions, &unions, sizeof unions, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = big_invalidate(c);
+    if (h.bad) return fail(CC_ERR_LABELS, "cc_load_labels: not a minimum-id labelling (need 0 <= l[v] <= v, l[l[v]] == l[v])");
+    e = cc::launch_adopt(labels, c->n, c->parent, c->ds, (unsigned long long)c->n - h.roots, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cc_load_labels: copy");
     c->flat = true;
@@ -1302,19 +1295,15 @@ cc_status cc_load_forest(cc_ctx* c, const int32_t* parent) {
     if (!parent || reinterpret_cast<uintptr_t>(parent) % 4) return fail(CC_ERR_ARG, "cc_load_forest: null or misaligned");
     if (c->G > 1 || by_size(c)) return fail(CC_ERR_UNSUPPORTED, "cc_load_forest needs the default link rule on a plain handle");
     CC_DEVICE(c);
-    cudaError_t e = cudaMemsetAsync(&c->ds->labels_bad, 0, sizeof(unsigned), c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&c->ds->roots, 0, sizeof(unsigned long long), c->stream);
+    cudaError_t e = cudaMemsetAsync(&c->ds->checked, 0, sizeof(cc::DevState::Checked), c->stream);
     if (e == cudaSuccess) e = cc::launch_validate_forest(parent, c->n, c->ds, c->stream);
-    cc::DevState h;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, c->ds, sizeof h, cudaMemcpyDeviceToHost, c->stream);
+    cc::DevState::Checked h;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, &c->ds->checked, sizeof h, cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cc_load_forest: validate");
     c->launches[CC_K_LOAD]++;
-    if (h.labels_bad) return fail(CC_ERR_LABELS, "cc_load_forest: need 0 <= parent[v] <= v");
-    unsigned long long unions = (unsigned long long)c->n - h.roots;
-    e = cudaMemcpyAsync(c->parent, parent, sizeof(int) * (size_t)c->n, cudaMemcpyDeviceToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&c->ds->unions, &unions, sizeof unions, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = big_invalidate(c);
+    if (h.bad) return fail(CC_ERR_LABELS, "cc_load_forest: need 0 <= parent[v] <= v");
+    e = cc::launch_adopt(parent, c->n, c->parent, c->ds, (unsigned long long)c->n - h.roots, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cc_load_forest: copy");
     c->flat = false;

@@ -17,10 +17,12 @@ enum : unsigned {
 // Device-side bookkeeping of one handle (one small allocation).
 struct DevState {
     unsigned status;            // ST_* bits, cleared by cc_sync
-    unsigned labels_bad;        // set by the label validator
-    unsigned long long unions;  // successful hooks since create / reset
-    unsigned long long roots;   // roots counted by the label validator
     unsigned queue;             // work-queue counter of the batched form
+    unsigned long long unions;  // successful hooks since create / reset
+    struct Checked {            // what the validators found
+        unsigned long long roots;
+        unsigned bad;
+    } checked;
     unsigned max_depth;         // forest height diagnostic
     unsigned long long sum_depth;
     int big_root;               // largest-component filter: the root R whose tree the bitmap
@@ -318,5 +320,12 @@ cudaError_t launch_validate_forest(const int* p, int64_t n, DevState* ds, cudaSt
 
 // Checks 0 <= lab[v] <= v and lab[lab[v]] == lab[v]; counts roots.
 cudaError_t launch_validate_labels(const int* lab, int64_t n, DevState* ds, cudaStream_t s);
+
+// parent = the validated array src; also sets ds->unions and turns the
+// largest-component filter off.
+cudaError_t launch_adopt(const int* src, int64_t n, int* parent, DevState* ds, unsigned long long unions,
+                         cudaStream_t s);
+// out (16-byte aligned) = parent.
+cudaError_t launch_copy_ids(const int* parent, int64_t n, int* out, bool pdl, cudaStream_t s);
 
 }  // namespace cc

@@ -41,7 +41,12 @@ def test_validation_counts_roots_and_finds_each_fault(cc, n, shift):
     f = cc.Forest(n)
     f.load_labels(dev(lab, shift))
     assert f.components() == int((lab == np.arange(n)).sum())
-    assert np.array_equal(f.labels().cpu().numpy(), lab)
+    for at in (0, 1):                           # flat: copied; into any 4-byte-aligned place
+        out = torch.full((n + 2,), -7, dtype=torch.int32, device="cuda")
+        f.labels(out[at:at + n])
+        assert np.array_equal(out[at:at + n].cpu().numpy(), lab) and int(out[n + at:].max()) == -7
+    f.load_forest(dev(lab, shift))
+    assert np.array_equal(f.labels().cpu().numpy(), lab)        # not known to be flat
     f.load_forest(dev(lab, shift))
     assert f.components() == int((lab == np.arange(n)).sum())
     for v in {0, n // 2, n - 1}:                # one id above its own place, or negative
