@@ -1338,39 +1338,53 @@ cudaError_t launch_compress_touched(int* parent, int n, const int* edges, int64_
 
 // Checks an array loaded from outside and counts its roots: LABELS wants
 // 0 <= a[v] <= v and a[a[v]] == a[v], else only 0 <= a[v] <= v. Bound by the
-// stream of n ids plus, for labels, the gather of each label's own label
-// (skipped at a root; one hot line where a giant component holds most ids).
-// Four ids per thread and step (one 16-byte load where the array allows it),
-// a grid of resident CTAs, and ONE atomic per CTA on the root counter: with
-// one per warp, 2^25 ids queued 2^20 atomics on that word and the pass took
-// 668 us; now 49 us (events around it; 128 MB: 2.7 TB/s).
+// stream of n ids plus, for labels, the gather of each label's own label (one
+// hot line where a giant component holds most ids). Each thread has four
+// quadruples, whose loads (16 bytes where the array allows it) and then gathers
+// are all in flight together, and a CTA makes ONE atomic on the root counter:
+// with one per warp, 2^25 ids queued 2^20 atomics on that word and the pass took
+// 668 us; on a resident grid with a quadruple per thread and step 49; now 35.
 template <bool LABELS>
 __global__ void __launch_bounds__(256)
 k_validate(const int* __restrict__ a, int64_t n, int vec, DevState* __restrict__ ds) {
     __shared__ int part[8];
+    constexpr int Q = 4;
+    const int64_t first = (int64_t)blockIdx.x * (256 * 4 * Q);
     int roots = 0;
     bool bad = false;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t v0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; v0 < n; v0 += stride) {
-        int x[4];
-        if (vec && v0 + 4 <= n) {
-            const int4 q = *reinterpret_cast<const int4*>(a + v0);
-            x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
-        } else {
+    if (vec && first + 256 * 4 * Q <= n) {
+        int x[Q][4], y[Q][4];
+        const int v0 = (int)first + 4 * (int)threadIdx.x;
 #pragma unroll
-            for (int i = 0; i < 4; i++) x[i] = v0 + i < n ? a[v0 + i] : 0;  // past n: 0 <= 0, not counted
+        for (int j = 0; j < Q; j++) {
+            const int4 q = *reinterpret_cast<const int4*>(a + v0 + 1024 * j);
+            x[j][0] = q.x; x[j][1] = q.y; x[j][2] = q.z; x[j][3] = q.w;
         }
-        int y[4];
+        if (LABELS) {
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const bool in = x[i] >= 0 && (int64_t)x[i] <= v0 + i;
-            bad |= !in;
-            y[i] = LABELS && in && v0 + i < n && (int64_t)x[i] != v0 + i ? a[x[i]] : x[i];
+            for (int j = 0; j < Q; j++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const int v = v0 + 1024 * j + i;
+                    y[j][i] = a[(unsigned)x[j][i] < (unsigned)v ? x[j][i] : v];  // stays in range
+                }
         }
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            bad |= y[i] != x[i];
-            roots += v0 + i < n && (int64_t)x[i] == v0 + i;
+        for (int j = 0; j < Q; j++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const int v = v0 + 1024 * j + i;
+                bad |= (unsigned)x[j][i] > (unsigned)v || (LABELS && y[j][i] != x[j][i]);
+                roots += x[j][i] == v;
+            }
+    } else {
+        for (int j = 0; j < Q * 4; j++) {
+            const int64_t v = first + 256 * j + threadIdx.x;
+            if (v >= n) break;
+            const int x = a[v];
+            const bool in = x >= 0 && (int64_t)x <= v;
+            bad |= !in || (LABELS && a[x] != x);
+            roots += (int64_t)x == v;
         }
     }
     if (bad) atomicOr(&ds->checked.bad, 1u);
@@ -1386,10 +1400,7 @@ k_validate(const int* __restrict__ a, int64_t n, int vec, DevState* __restrict__
 
 template <bool LABELS>
 static cudaError_t validate(const int* a, int64_t n, DevState* ds, cudaStream_t s) {
-    int64_t g = (n + 1023) / 1024;
-    const int64_t cap = resident_grid<k_validate<LABELS>>(256);
-    if (g > cap) g = cap;
-    k_validate<LABELS><<<(unsigned)g, 256, 0, s>>>(a, n, pair_vec(a) == 2, ds);
+    k_validate<LABELS><<<blocks_for(n, 4096), 256, 0, s>>>(a, n, pair_vec(a) == 2, ds);
     return cudaGetLastError();
 }
 
