@@ -292,3 +292,55 @@ def test_batched_operations_of_all_lengths(cc, opts):
     with pytest.raises(cc.CCError) as ex:
         f.sync()
     assert ex.value.status == cc.CC_ERR_RANGE
+
+
+# ------------------------------------------------------- captured and replayed
+
+@pytest.mark.parametrize("opts", [{}, {"pdl": 2, "compress_every": 2, "big_filter": 100, "edge_order": 6},
+                                  {"pdl": 0, "compress_every": 0, "query_halving": 1}])
+@pytest.mark.parametrize("n,k", [(3000, 1000), (200_000, 300_000)])
+def test_a_captured_pass_replays_on_new_inputs(cc, opts, n, k):
+    """The dependent launches, the small update, the tiles, Bulk-Find and the
+    label copy inside a CUDA graph, replayed after the inputs have changed."""
+    import oracle
+    r = np.random.default_rng(n)
+    st = torch.cuda.Stream()
+    edges = [torch.empty((k, 2), dtype=torch.int32, device="cuda") for _ in range(3)]
+    pairs = torch.empty((5000, 2), dtype=torch.int32, device="cuda")
+    out = torch.empty((3, 5000), dtype=torch.uint8, device="cuda")
+    found = torch.empty(10000, dtype=torch.int32, device="cuda")
+    labels = torch.empty(n, dtype=torch.int32, device="cuda")
+    f = cc.Forest(n, stream=st, **opts)
+
+    def fill():
+        for e in edges:
+            e.copy_(torch.from_numpy(r.integers(0, n, size=(k, 2)).astype(np.int32)))
+        pairs.copy_(torch.from_numpy(r.integers(0, n, size=(5000, 2)).astype(np.int32)))
+        torch.cuda.synchronize()
+
+    def one_pass():
+        f.reset()
+        for e, o in zip(edges, out):
+            f.bulk_update(e)
+            f.bulk_query(pairs, o)
+        f.bulk_find(pairs.view(-1), found)
+        f.labels(labels)
+
+    fill()
+    one_pass()                              # scratch of the first calls
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        one_pass()
+    for _ in range(2):
+        fill()
+        g.replay()
+        torch.cuda.synchronize()
+        ref = oracle.OracleUF(n)
+        q = pairs.cpu().numpy()
+        for e, o in zip(edges, out):
+            ref.bulk_update(e.cpu().numpy())
+            assert np.array_equal(o.cpu().numpy(), ref.bulk_query(q))
+        assert np.array_equal(labels.cpu().numpy(), ref.labels())
+        assert np.array_equal(found.cpu().numpy(), ref.labels()[q.reshape(-1)])
+        f.sync()
