@@ -69,7 +69,9 @@ typedef enum {
 /* Tunables (cc_set_option / cc_get_option). */
 typedef enum {
     CC_OPT_BLOCK = 0,            /* threads per block for the bulk kernels: 64..1024, multiple of 32 (default 256) */
-    CC_OPT_EDGES_PER_THREAD = 1, /* edges (or pairs) per thread in update and query: 1, 2 or 4 (default 2) */
+    CC_OPT_EDGES_PER_THREAD = 1, /* edges (or pairs) per thread in update and query: 1, 2 or 4
+                                    (default 2); CC_OPT_UPDATE_VARIANT 0 and CC_OPT_QUERY_VARIANT 0
+                                    take fewer where that leaves an SM without work */
     CC_OPT_COMPRESS_EVERY = 2,   /* cc_bulk_update compresses after every c-th call; 0 = never (default 1) */
     CC_OPT_COMPRESS_SCOPE = 3,   /* scope of that automatic compression: a cc_compress_scope (default ALL) */
     CC_OPT_QUERY_HALVING = 4,    /* how Bulk-Query finds walk (all pairs of a thread in lockstep): 0

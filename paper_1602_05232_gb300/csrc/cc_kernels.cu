@@ -15,6 +15,22 @@ static inline unsigned blocks_for(int64_t work, int64_t per_block) {
     return (unsigned)((work + per_block - 1) / per_block);
 }
 
+// Edges (pairs) per thread of a launch with one chunk per thread: as many as
+// asked for, but not so many that an SM is left without a CTA. Default options
+// (2 per thread, 256 threads), 2 and 1 per thread: minibatches of up to 2^18,
+// 30,000 on average, on 10^6 vertices with 50,001 pairs asked after each 894 and
+// 854 us for 104 steps; but 434 and 473 for 32 of 2^17, which fill the chip.
+static int spread(int ept, int64_t k, int block) {
+    thread_local int sms[16] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    int own = 0;
+    int& n = dev >= 0 && dev < 16 ? sms[dev] : own;
+    if (!n) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    while (ept > 1 && k < (int64_t)ept * block * n) ept /= 2;
+    return ept;
+}
+
 // ------------------------------------------------------------------ reset
 
 // parent[v] = v: n singletons, the empty graph G_0, with no links made and no
@@ -701,6 +717,8 @@ cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevSt
     if (cfg.variant == 0 && k >= kTileEdges) {
         cfg.variant = 5;
         cfg.block = 128;
+    } else if (cfg.variant == 0) {
+        cfg.ept = spread(cfg.ept, k, cfg.block);
     }
 #define CC_UPD(E, P) update_inst<E, P>(edges, k, vec, parent, n, ds, cfg.block, cfg.window, cfg.pdl, cfg.hook, cfg.variant ? cfg.warphook : 0, BigArgs{cfg.big, cfg.alt}, s)
     switch (cfg.variant * 8 + cfg.ept) {
@@ -1071,6 +1089,7 @@ cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_
         return cudaGetLastError();
     }
     if (cfg.qept) cfg.ept = cfg.qept;
+    if (cfg.query_variant == 0) cfg.ept = spread(cfg.ept, k, cfg.block);
     const int vec = pair_vec(pairs);
     const int ovec = (reinterpret_cast<uintptr_t>(out) % cfg.ept) == 0;
     const unsigned g = blocks_for(k, (int64_t)cfg.ept * cfg.block);

@@ -160,7 +160,8 @@ def test_query_walks_answer_as_the_roots_do(cc, k, shape):
     q[2::11, 1] = root[q[2::11, 0]]
     want = (root[q[:, 0]] == root[q[:, 1]]).astype(np.uint8)
     for mode in (0, 1, 2):
-        for extra in ({}, {"query_pairs_per_thread": 1}, {"query_pairs_per_thread": 4, "query_variant": 1}):
+        for extra in ({}, {"query_pairs_per_thread": 1}, {"query_pairs_per_thread": 4, "query_variant": 1},
+                      {"query_pairs_per_thread": 4, "block": 64}):
             f = cc.Forest(n, query_halving=mode, **extra)
             if shape == "flat":
                 f.load_labels(dev(root))
