@@ -493,7 +493,8 @@ cc_status cc_copy_nonloop(cc_ctx* ctx, int32_t* out, int64_t cap, int64_t* count
  * `res`: device, k int32 (it may be `S` itself). One cooperative kernel, or two
  * kernels when the forest is known to be flat (right after a full compression,
  * with no update since). Asynchronous, but for the scratch (12 bytes per vertex
- * of the largest S so far) allocated on first use and grown. */
+ * of the largest S so far) allocated on first use and grown. CC_ERR_CUDA, with
+ * nothing enqueued, on a stream that is capturing. */
 cc_status cc_bulk_find(cc_ctx* ctx, const int32_t* S, int64_t k, int32_t* res);
 
 /* For the last Bulk-Find: the number of traversed non-root vertices

@@ -235,6 +235,8 @@ void bulk_find_free(BulkFindState& b) {
 
 static cudaError_t launch(BulkFindState& b, int* parent, int n, const int* S, int64_t k, int* res,
                           uint8_t* out, DevState* ds, bool flat, bool pdl, cudaStream_t s) {
+    // A graph would keep this call's stamp, and buffers that a larger call frees.
+    if (capturing(s)) return cudaErrorStreamCaptureUnsupported;
     cudaError_t e = cudaSuccess;
     if (!b.mark) {
         BulkFindCounters* count = nullptr;

@@ -131,6 +131,17 @@ static void launch_windowed(void (*kernel)(Params...), unsigned grid, int block,
     launch_windowed_smem(kernel, grid, block, 0, s, window, pdl, args...);
 }
 
+// Whether work given to s is recorded into a graph instead of run (or may be:
+// the query fails on the legacy stream during another stream's capture).
+static inline bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Alignment class of a pair array: 2 = 16-byte, 1 = 8-byte, 0 = 4-byte.
 int pair_vec(const void* p);
 

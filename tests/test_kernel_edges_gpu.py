@@ -301,15 +301,14 @@ def test_batched_operations_of_all_lengths(cc, opts):
                                   {"pdl": 0, "compress_every": 0, "query_halving": 1}])
 @pytest.mark.parametrize("n,k", [(3000, 1000), (200_000, 300_000)])
 def test_a_captured_pass_replays_on_new_inputs(cc, opts, n, k):
-    """The dependent launches, the small update, the tiles, Bulk-Find and the
-    label copy inside a CUDA graph, replayed after the inputs have changed."""
+    """The dependent launches, the small update and the tiles inside a CUDA
+    graph, replayed after the inputs have changed."""
     import oracle
     r = np.random.default_rng(n)
     st = torch.cuda.Stream()
     edges = [torch.empty((k, 2), dtype=torch.int32, device="cuda") for _ in range(3)]
     pairs = torch.empty((5000, 2), dtype=torch.int32, device="cuda")
     out = torch.empty((3, 5000), dtype=torch.uint8, device="cuda")
-    found = torch.empty(10000, dtype=torch.int32, device="cuda")
     labels = torch.empty(n, dtype=torch.int32, device="cuda")
     f = cc.Forest(n, stream=st, **opts)
 
@@ -324,7 +323,6 @@ def test_a_captured_pass_replays_on_new_inputs(cc, opts, n, k):
         for e, o in zip(edges, out):
             f.bulk_update(e)
             f.bulk_query(pairs, o)
-        f.bulk_find(pairs.view(-1), found)
         f.labels(labels)
 
     fill()
@@ -343,5 +341,30 @@ def test_a_captured_pass_replays_on_new_inputs(cc, opts, n, k):
             ref.bulk_update(e.cpu().numpy())
             assert np.array_equal(o.cpu().numpy(), ref.bulk_query(q))
         assert np.array_equal(labels.cpu().numpy(), ref.labels())
-        assert np.array_equal(found.cpu().numpy(), ref.labels()[q.reshape(-1)])
         f.sync()
+
+
+def test_bulk_find_is_refused_under_capture(cc):
+    """Its scratch may be freed by a later, larger call, and its stamp is the call's."""
+    st = torch.cuda.Stream()
+    f = cc.Forest(5000, stream=st)
+    ids = torch.arange(5000, dtype=torch.int32, device="cuda")
+    e = torch.tensor([[1, 2], [2, 3]], dtype=torch.int32, device="cuda")
+    found = torch.empty_like(ids)
+    out = torch.empty(2, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    f.bulk_find(ids, found)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        with pytest.raises(cc.CCError) as ex:
+            f.bulk_find(ids, found)
+        assert ex.value.status == cc.CC_ERR_CUDA
+        f.bulk_update(e)
+        f.bulk_query(e, out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert out.tolist() == [1, 1] and f.components() == 4998
+    f.bulk_find(ids[:4], found[:4])
+    torch.cuda.synchronize()
+    assert found[:4].tolist() == [0, 1, 1, 1]
