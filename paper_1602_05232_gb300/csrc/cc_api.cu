@@ -117,6 +117,8 @@ struct cc_ctx {
     std::vector<cudaEvent_t> spare;
     uint64_t update_calls = 0;
     bool flat = true;  // every tree has height <= 1
+    bool replayable = false;  // a caller's graph holds a Bulk-Update of this forest that leaves it not
+                              // flat, and may replay it at any time
     cudaAccessPolicyWindow window = {};  // L2 window over parent (num_bytes 0 = off)
 
     // batched form
@@ -256,6 +258,19 @@ cc_status do_compress(cc_ctx* c, int scope, const int32_t* edges, int64_t k) {
 bool compress_due(const cc_ctx* c) {
     const int64_t every = c->opt[CC_OPT_COMPRESS_EVERY];
     return every > 0 && (c->update_calls + 1) % (uint64_t)every == 0;
+}
+
+// The forest is no longer known to be flat.
+void not_flat(cc_ctx* c) {
+    c->flat = false;
+    if (!c->replayable) c->replayable = cc::capturing(c->stream);
+}
+
+// Whether the forest is flat for certain when the work enqueued next runs. A
+// graph that holds an update makes `flat` out of date when it is replayed, and
+// recorded work runs on whatever the forest is by then.
+bool surely_flat(const cc_ctx* c) {
+    return c->flat && !c->replayable && !cc::capturing(c->stream);
 }
 
 // Launch options of a Bulk-Update: CC_OPT_HOOK = 2 hooks with atomicMin only
@@ -444,7 +459,7 @@ cc_status paper_update(cc_ctx* c, const int32_t* edges, int64_t k) {
             c->bf.res = q;
             c->bf.cap_res = 2 * k;
         }
-        e = cc::bulk_find(c->bf, c->parent, (int)c->n, edges, 2 * k, c->bf.res, c->ds, c->flat,
+        e = cc::bulk_find(c->bf, c->parent, (int)c->n, edges, 2 * k, c->bf.res, c->ds, surely_flat(c),
                           c->opt[CC_OPT_PDL] != 0, c->stream);
         c->launches[CC_K_UPDATE] += c->bf.launches - before;
         if (e != cudaSuccess) return cuda_fail(e, "schedule 1: Bulk-Find relabel");
@@ -709,7 +724,8 @@ cc_status cc_bulk_update(cc_ctx* c, const int32_t* edges, int64_t k) {
         });
     }
     if (s != CC_OK) return s;
-    c->flat = false;
+    if (compress && c->opt[CC_OPT_COMPRESS_SCOPE] == CC_COMPRESS_ALL) c->flat = false;  // until the end of this call
+    else not_flat(c);
     c->update_calls++;
     if (compress)
         return do_compress(c, (int)c->opt[CC_OPT_COMPRESS_SCOPE], given, k);  // a set: same endpoints
@@ -726,7 +742,7 @@ cc_status cc_bulk_query(cc_ctx* c, const int32_t* pairs, int64_t k, uint8_t* out
     if (c->opt[CC_OPT_BULK_FIND] == 1) {
         const uint64_t before = c->bf.launches;
         s = run(c, CC_K_QUERY, "bulk_query(Bulk-Find)", [&] {
-            return cc::bulk_find_query(c->bf, c->parent, (int)c->n, pairs, k, out, c->ds, c->flat,
+            return cc::bulk_find_query(c->bf, c->parent, (int)c->n, pairs, k, out, c->ds, surely_flat(c),
                                        c->opt[CC_OPT_PDL] != 0, c->stream);
         });
         c->launches[CC_K_QUERY] += c->bf.launches - before - 1;  // run() counted one
@@ -779,7 +795,7 @@ cc_status cc_labels(cc_ctx* c, int32_t* out) {
         return s;
     }
     // flat already: the parents are the labels
-    const bool copy = c->flat && reinterpret_cast<uintptr_t>(out) % 16 == 0;
+    const bool copy = surely_flat(c) && reinterpret_cast<uintptr_t>(out) % 16 == 0;
     cc_status s = run(c, CC_K_LABELS, "labels", [&] {
         if (copy) return cc::launch_copy_ids(c->parent, c->n, out, c->opt[CC_OPT_PDL] != 0, c->stream);
         return cc::launch_compress_all(c->parent, c->n, out, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream);
@@ -1057,7 +1073,7 @@ cc_status cc_submit(cc_ctx* c, const cc_op* ops, int64_t nops) {
         c->staging_pending[j] = true;
         c->stage = j ^ 1;
     }
-    c->flat = false;
+    not_flat(c);
     c->fresh = false;
     return st;
 }
@@ -1267,7 +1283,7 @@ cc_status cc_bulk_find(cc_ctx* c, const int32_t* S, int64_t k, int32_t* res) {
         return fail(CC_ERR_ARG, "cc_bulk_find: arrays must be 4-byte aligned");
     CC_DEVICE(c);
     const uint64_t before = c->bf.launches;
-    cudaError_t e = cc::bulk_find(c->bf, c->parent, (int)c->n, S, k, res, c->ds, c->flat,
+    cudaError_t e = cc::bulk_find(c->bf, c->parent, (int)c->n, S, k, res, c->ds, surely_flat(c),
                                   c->opt[CC_OPT_PDL] != 0, c->stream);
     c->launches[CC_K_QUERY] += c->bf.launches - before;
     if (e != cudaSuccess) return cuda_fail(e, "cc_bulk_find");

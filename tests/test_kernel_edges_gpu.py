@@ -344,6 +344,62 @@ def test_a_captured_pass_replays_on_new_inputs(cc, opts, n, k):
         f.sync()
 
 
+@pytest.mark.parametrize("recorded", ["update", "labels"])
+@pytest.mark.parametrize("n,k", [(3000, 1000), (200_000, 60_000)])
+def test_labels_and_bulk_find_do_not_trust_a_forest_that_a_graph_changes(cc, recorded, n, k):
+    """A replayed update changes a forest that the handle last saw compressed,
+    and recorded labels run on a forest that was updated since: neither may
+    take the copy of, or the short Bulk-Find on, a flat forest."""
+    import oracle
+    r = np.random.default_rng(n + k)
+    st = torch.cuda.Stream()
+    e = torch.empty((k, 2), dtype=torch.int32, device="cuda")
+    labels = torch.empty(n, dtype=torch.int32, device="cuda")
+    ids = torch.arange(n, dtype=torch.int32, device="cuda")
+    found = torch.empty_like(ids)
+    f = cc.Forest(n, stream=st, compress_every=0, update_variant=1)
+    ref = oracle.OracleUF(n)
+
+    def fill():
+        # a path through the ids in steps of random length: deep trees
+        x = np.sort(r.choice(n, size=k + 1, replace=False)).astype(np.int32)
+        p = np.stack([x[1:], x[:-1]], axis=1)
+        e.copy_(torch.from_numpy(p))
+        torch.cuda.synchronize()
+        ref.bulk_update(p)
+
+    def check():
+        torch.cuda.synchronize()
+        assert np.array_equal(labels.cpu().numpy(), ref.labels())
+
+    fill()
+    f.bulk_update(e)
+    f.labels(labels)        # flat from here, as the handle sees it
+    f.bulk_find(ids, found)
+    check()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        f.bulk_update(e) if recorded == "update" else f.labels(labels)
+    for _ in range(3):
+        fill()
+        if recorded == "update":
+            g.replay()
+            torch.cuda.synchronize()
+            f.bulk_find(ids, found)
+            torch.cuda.synchronize()
+            assert np.array_equal(found.cpu().numpy(), ref.labels())
+            fill()
+            g.replay()
+            torch.cuda.synchronize()
+            f.labels(labels)
+        else:
+            f.bulk_update(e)
+            torch.cuda.synchronize()
+            g.replay()
+        check()
+    f.sync()
+
+
 def test_bulk_find_is_refused_under_capture(cc):
     """Its scratch may be freed by a later, larger call, and its stamp is the call's."""
     st = torch.cuda.Stream()
