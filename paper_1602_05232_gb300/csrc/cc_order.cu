@@ -93,7 +93,8 @@ k_order_count(const int* __restrict__ edges, int64_t k, int vec, int n, int shif
               int* __restrict__ totals, int early, const unsigned* big, const DevState* ds) {
     __shared__ int hist[kMaxBuckets];
     pdl_trigger();
-    if (big && ds->big_root >= 0) {  // the update reads the caller's order (BigArgs)
+    // read before the wait, so past L1: the kernel before may be the reset that wrote it
+    if (big && *(volatile const int*)&ds->big_root >= 0) {  // the update reads the caller's order (BigArgs)
         pdl_wait();                // still complete only after the kernel before
         return;
     }
