@@ -748,16 +748,13 @@ cc_status cc_bulk_query(cc_ctx* c, const int32_t* pairs, int64_t k, uint8_t* out
         c->launches[CC_K_QUERY] += c->bf.launches - before - 1;  // run() counted one
         return s;
     }
-    if (by_size(c)) {
-        const bool flat = c->flat;
-        s = run(c, CC_K_QUERY, "bulk_query(generic)", [&] {
+    const bool flat = surely_flat(c);
+    if (by_size(c))
+        return run(c, CC_K_QUERY, "bulk_query(generic)", [&] {
             return cc::launch_query_generic(c->parent, (int)c->n, pairs, k, out, c->ds, flat,
                                             (int)c->opt[CC_OPT_BLOCK], c->stream);
         });
-        if (s == CC_OK && !flat) c->flat = false;
-        return s;
-    }
-    const int mode = c->flat ? 2 : c->opt[CC_OPT_QUERY_HALVING] != 0 ? 1 : 0;
+    const int mode = flat ? 2 : c->opt[CC_OPT_QUERY_HALVING] != 0 ? 1 : 0;
     s = run(c, CC_K_QUERY, "bulk_query", [&] {
         return cc::launch_query(c->parent, (int)c->n, pairs, k, out, c->ds, mode, cfg_of(c), c->stream);
     });

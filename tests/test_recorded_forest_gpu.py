@@ -1,0 +1,86 @@
+"""What a handle may know about a forest that CUDA graphs read and change:
+work that is only recorded has not run, and a graph may be replayed at any time."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+M = 1000                # groups of four vertices
+N = 4 * M
+
+
+@pytest.fixture(scope="module")
+def cc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1602_05232_gb300 import _build, cc as ccmod
+    _build.build_cc()
+    ccmod.load()
+    return ccmod
+
+
+def groups(*ij):
+    """The pairs (4g + i, 4g + j) of every group g, on the device."""
+    base = 4 * np.arange(M)[:, None, None] + np.array(ij)[None]
+    return torch.from_numpy(base.reshape(-1, 2).astype(np.int32)).cuda()
+
+
+def deepen(f, e):
+    """Joins each group by two updates that leave vertex 3 two links below its root."""
+    f.bulk_update(e[0])
+    f.bulk_update(e[1])
+
+
+def edges():
+    return groups((0, 1), (2, 3)), groups((1, 3))
+
+
+def all_pairs():
+    return groups((0, 1), (0, 2), (0, 3), (1, 2), (1, 3), (2, 3))
+
+
+ROOTS = np.repeat(4 * np.arange(M), 4)
+
+
+def record(st, fn):
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        fn()
+    return g
+
+
+def test_query_after_the_replay_of_an_update(cc):
+    """The forest was reset, then a graph made it deep."""
+    st = torch.cuda.Stream()
+    e, q = edges(), all_pairs()
+    out = torch.zeros(q.shape[0], dtype=torch.uint8, device="cuda")
+    f = cc.Forest(N, stream=st, compress_every=0, update_variant=1)
+    torch.cuda.synchronize()
+    g = record(st, lambda: deepen(f, e))
+    f.reset()
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    f.bulk_query(q, out)
+    torch.cuda.synchronize()
+    assert out.all()
+
+
+@pytest.mark.parametrize("link", [0, 1])
+def test_recorded_query_on_a_forest_that_is_deep_by_then(cc, link):
+    """A query recorded while the forest was flat, replayed after updates."""
+    st = torch.cuda.Stream()
+    e, q = edges(), all_pairs()
+    out = torch.zeros(q.shape[0], dtype=torch.uint8, device="cuda")
+    f = cc.Forest(N, stream=st, compress_every=0, update_variant=1, link=link, update_schedule=link)
+    torch.cuda.synchronize()
+    f.compress()
+    g = record(st, lambda: f.bulk_query(q, out))
+    deepen(f, e)
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    assert out.all()
