@@ -116,9 +116,13 @@ struct cc_ctx {
     std::vector<Timed> pending;
     std::vector<cudaEvent_t> spare;
     uint64_t update_calls = 0;
-    bool flat = true;  // every tree has height <= 1
-    bool replayable = false;  // a caller's graph holds a Bulk-Update of this forest that leaves it not
-                              // flat, and may replay it at any time
+    // What is known of the forest. Work that is only recorded into a caller's graph
+    // has not run, so it says nothing about `flat`; and the graph may be replayed at
+    // any time, with the forest left as the graph's last work on it leaves it.
+    bool flat = true;                // every tree has height <= 1 after the work that was run
+    unsigned long long rec_id = 0;   // the last capture that recorded such work (0: none)
+    bool rec_flat = false;           // every tree has height <= 1 after what it has recorded
+    bool replayable = false;         // an earlier capture left the forest not known to be flat
     cudaAccessPolicyWindow window = {};  // L2 window over parent (num_bytes 0 = off)
 
     // batched form
@@ -225,13 +229,50 @@ cc_status check_pairs(const int32_t* p, int64_t k, const char* name) {
     return CC_OK;
 }
 
+// Where work given to the stream goes: 0, it is run; else the id of the capture
+// that records it (kUnknown: the runtime does not say).
+constexpr unsigned long long kUnknown = ~0ull;
+unsigned long long capture_of(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return kUnknown;
+    }
+    return st == cudaStreamCaptureStatusNone ? 0 : st == cudaStreamCaptureStatusActive ? id : kUnknown;
+}
+
+// The work just given to the stream leaves the forest flat, or not known to be.
+void set_flat(cc_ctx* c, bool flat) {
+    const unsigned long long id = capture_of(c->stream);
+    if (id == 0) {
+        c->flat = flat;
+        return;
+    }
+    if (id != c->rec_id) {
+        c->replayable |= c->rec_id != 0 && !c->rec_flat;
+        c->rec_id = id;
+    }
+    c->rec_flat = flat && id != kUnknown;
+}
+
+// Whether the forest is flat for certain when the work given next runs: for work
+// that is run, after everything run before and whatever graph was replayed since;
+// for work that is recorded, after what its own capture has recorded before it.
+bool surely_flat(const cc_ctx* c) {
+    if (!c->flat && !c->rec_flat) return false;
+    const unsigned long long id = capture_of(c->stream);
+    if (id == 0) return c->flat && !c->replayable && (c->rec_id == 0 || c->rec_flat);
+    return id == c->rec_id && c->rec_flat;
+}
+
 cc_status do_compress(cc_ctx* c, int scope, const int32_t* edges, int64_t k) {
     if (c->opt[CC_OPT_LINK] == 1) {  // union by size: only the full generic pass
         cc_status s = run(c, CC_K_COMPRESS_ALL, "compress(all, generic)", [&] {
             return cc::launch_compress_generic(c->parent, c->n, nullptr, nullptr, c->ds,
                                                (int)c->opt[CC_OPT_BLOCK], c->stream);
         });
-        if (s == CC_OK) c->flat = true;
+        if (s == CC_OK) set_flat(c, true);
         return s;
     }
     if (scope == CC_COMPRESS_ALL) {
@@ -245,7 +286,7 @@ cc_status do_compress(cc_ctx* c, int scope, const int32_t* edges, int64_t k) {
         cc_status s = run(c, CC_K_COMPRESS_ALL, "compress(all)", [&] {
             return cc::launch_compress_all(c->parent, c->n, nullptr, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream, big);
         });
-        if (s == CC_OK) c->flat = true;
+        if (s == CC_OK) set_flat(c, true);
         return s;
     }
     if (k == 0) return CC_OK;
@@ -258,19 +299,6 @@ cc_status do_compress(cc_ctx* c, int scope, const int32_t* edges, int64_t k) {
 bool compress_due(const cc_ctx* c) {
     const int64_t every = c->opt[CC_OPT_COMPRESS_EVERY];
     return every > 0 && (c->update_calls + 1) % (uint64_t)every == 0;
-}
-
-// The forest is no longer known to be flat.
-void not_flat(cc_ctx* c) {
-    c->flat = false;
-    if (!c->replayable) c->replayable = cc::capturing(c->stream);
-}
-
-// Whether the forest is flat for certain when the work enqueued next runs. A
-// graph that holds an update makes `flat` out of date when it is replayed, and
-// recorded work runs on whatever the forest is by then.
-bool surely_flat(const cc_ctx* c) {
-    return c->flat && !c->replayable && !cc::capturing(c->stream);
 }
 
 // Launch options of a Bulk-Update: CC_OPT_HOOK = 2 hooks with atomicMin only
@@ -665,7 +693,7 @@ cc_status cc_reset(cc_ctx* c) {
         return cc::launch_reset(c->parent, c->n, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream);
     });
     if (s == CC_OK) {
-        c->flat = true;
+        set_flat(c, true);
         c->update_calls = 0;
         c->fresh = true;
         if (c->size) {
@@ -696,7 +724,7 @@ cc_status cc_bulk_update(cc_ctx* c, const int32_t* edges, int64_t k) {
         });
         if (s != CC_OK) return s;
         c->fresh = false;
-        c->flat = true;  // the kernel leaves it so: no compression is due
+        set_flat(c, true);  // the kernel leaves it so: no compression is due
         c->update_calls++;
         return CC_OK;
     }
@@ -724,12 +752,12 @@ cc_status cc_bulk_update(cc_ctx* c, const int32_t* edges, int64_t k) {
         });
     }
     if (s != CC_OK) return s;
-    if (compress && c->opt[CC_OPT_COMPRESS_SCOPE] == CC_COMPRESS_ALL) c->flat = false;  // until the end of this call
-    else not_flat(c);
     c->update_calls++;
-    if (compress)
-        return do_compress(c, (int)c->opt[CC_OPT_COMPRESS_SCOPE], given, k);  // a set: same endpoints
-    return CC_OK;
+    const bool full = compress && (c->opt[CC_OPT_COMPRESS_SCOPE] == CC_COMPRESS_ALL || by_size(c));
+    if (!full) set_flat(c, false);
+    if (compress) s = do_compress(c, (int)c->opt[CC_OPT_COMPRESS_SCOPE], given, k);  // a set: same endpoints
+    if (full && s != CC_OK) set_flat(c, false);
+    return s;
 }
 
 cc_status cc_bulk_query(cc_ctx* c, const int32_t* pairs, int64_t k, uint8_t* out) {
@@ -788,7 +816,7 @@ cc_status cc_labels(cc_ctx* c, int32_t* out) {
             return cc::launch_compress_generic(c->parent, c->n, out, c->comp, c->ds,
                                                (int)c->opt[CC_OPT_BLOCK], c->stream);
         });
-        if (s == CC_OK) c->flat = true;
+        if (s == CC_OK) set_flat(c, true);
         return s;
     }
     // flat already: the parents are the labels
@@ -797,7 +825,7 @@ cc_status cc_labels(cc_ctx* c, int32_t* out) {
         if (copy) return cc::launch_copy_ids(c->parent, c->n, out, c->opt[CC_OPT_PDL] != 0, c->stream);
         return cc::launch_compress_all(c->parent, c->n, out, c->ds, (int)c->opt[CC_OPT_BLOCK], c->opt[CC_OPT_PDL] != 0, c->stream);
     });
-    if (s == CC_OK) c->flat = true;
+    if (s == CC_OK) set_flat(c, true);
     return s;
 }
 
@@ -1070,7 +1098,7 @@ cc_status cc_submit(cc_ctx* c, const cc_op* ops, int64_t nops) {
         c->staging_pending[j] = true;
         c->stage = j ^ 1;
     }
-    not_flat(c);
+    set_flat(c, false);
     c->fresh = false;
     return st;
 }

@@ -84,3 +84,85 @@ def test_recorded_query_on_a_forest_that_is_deep_by_then(cc, link):
     g.replay()
     torch.cuda.synchronize()
     assert out.all()
+
+
+RECORDED = {
+    "labels": lambda f, e: f.labels(),
+    "compress": lambda f, e: f.compress(),
+    "reset": lambda f, e: f.reset(),
+    "small update": lambda f, e: f.bulk_update(e[0]),
+    "compressing update": lambda f, e: f.bulk_update(e[0]),
+    "update, then compress": lambda f, e: (deepen(f, e), f.compress()),
+}
+
+
+@pytest.mark.parametrize("ask", ["labels", "find", "query"])
+@pytest.mark.parametrize("recorded", RECORDED)
+def test_recorded_work_has_not_flattened_anything(cc, recorded, ask):
+    """A deep forest, work that flattens it recorded but not run, then a call."""
+    st = torch.cuda.Stream()
+    e, q = edges(), all_pairs()
+    out = torch.zeros(q.shape[0], dtype=torch.uint8, device="cuda")
+    ids = torch.arange(N, dtype=torch.int32, device="cuda")
+    f = cc.Forest(N, stream=st, compress_every=0, update_variant=1)
+
+    def check():
+        torch.cuda.synchronize()
+        if ask == "query":
+            out.zero_()
+            torch.cuda.synchronize()
+            f.bulk_query(q, out)
+            torch.cuda.synchronize()
+            assert out.all()
+        else:
+            got = f.labels() if ask == "labels" else f.bulk_find(ids)
+            torch.cuda.synchronize()
+            assert np.array_equal(got.cpu().numpy(), ROOTS)
+
+    torch.cuda.synchronize()
+    deepen(f, e)
+    assert f.depth()[0] == 2
+    f.set_option("update_variant", 0 if recorded == "small update" else 1)
+    f.set_option("compress_every", int(recorded == "compressing update"))
+    g = record(st, lambda: RECORDED[recorded](f, e))
+    check()
+    f.reset()
+    f.set_option("update_variant", 1)
+    f.set_option("compress_every", 0)
+    if recorded != "reset":
+        deepen(f, e)
+        torch.cuda.synchronize()
+        g.replay()
+        check()
+
+
+def test_recorded_calls_see_what_was_recorded_before_them(cc):
+    """Within one capture: flat after the compression, not before and not after
+    the next update, whatever the forest is when the graph is replayed."""
+    st = torch.cuda.Stream()
+    e, q = edges(), all_pairs()
+    outs = torch.zeros((3, q.shape[0]), dtype=torch.uint8, device="cuda")
+    labels = torch.empty((2, N), dtype=torch.int32, device="cuda")
+    f = cc.Forest(N, stream=st, compress_every=0, update_variant=1)
+    torch.cuda.synchronize()
+
+    def step():
+        f.bulk_query(q, outs[0])
+        f.compress()
+        f.bulk_query(q, outs[1])
+        f.labels(labels[0])
+        f.reset()
+        deepen(f, e)
+        f.bulk_query(q, outs[2])
+        f.labels(labels[1])
+
+    g = record(st, step)
+    for _ in range(2):
+        deepen(f, e)
+        outs.zero_()
+        labels.zero_()
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        assert outs.all()
+        assert np.array_equal(labels.cpu().numpy(), np.stack([ROOTS, ROOTS]))
