@@ -18,7 +18,10 @@ namespace {
 
 thread_local std::string g_err;
 
+// Leaves no error of the CUDA runtime behind, which the next launch of this
+// thread, of any handle, would report as its own.
 cc_status fail(cc_status s, const char* fmt, ...) {
+    if (s == CC_ERR_CUDA || s == CC_ERR_OOM) cudaGetLastError();
     char buf[512];
     va_list ap;
     va_start(ap, fmt);

@@ -2,6 +2,9 @@
 work that is only recorded has not run, and a graph may be replayed at any time."""
 from __future__ import annotations
 
+import contextlib
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -166,3 +169,34 @@ def test_recorded_calls_see_what_was_recorded_before_them(cc):
         torch.cuda.synchronize()
         assert outs.all()
         assert np.array_equal(labels.cpu().numpy(), np.stack([ROOTS, ROOTS]))
+
+
+@contextlib.contextmanager
+def foreign_capture():
+    """While a stream that the legacy stream synchronises with is captured, which
+    work given to the legacy stream is refused by and ends."""
+    try:
+        rt = ctypes.CDLL("libcudart.so." + torch.version.cuda.split(".")[0])
+    except OSError:
+        pytest.skip("no CUDA runtime library to create a blocking stream with")
+    st, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    assert rt.cudaStreamCreate(ctypes.byref(st)) == 0
+    assert rt.cudaStreamBeginCapture(st, 0) == 0
+    try:
+        yield
+    finally:
+        rt.cudaStreamEndCapture(st, ctypes.byref(graph))
+        rt.cudaGetLastError()
+        assert rt.cudaStreamDestroy(st) == 0
+
+
+def test_a_refused_call_does_not_fail_the_next(cc):
+    f = cc.Forest(N, stream=0)
+    labels = torch.zeros(N, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    with foreign_capture():
+        with pytest.raises(cc.CCError) as ex:
+            f.load_labels(labels)
+        assert ex.value.status == cc.CC_ERR_CUDA
+    f.compress()
+    assert f.components() == N
