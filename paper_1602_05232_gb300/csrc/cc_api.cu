@@ -233,9 +233,12 @@ cc_status check_pairs(const int32_t* p, int64_t k, const char* name) {
 }
 
 // Where work given to the stream goes: 0, it is run; else the id of the capture
-// that records it (kUnknown: the runtime does not say).
+// that records it (kUnknown: the runtime does not say). The legacy stream cannot
+// be captured, and asking about it fails while a stream that synchronises with
+// it is.
 constexpr unsigned long long kUnknown = ~0ull;
 unsigned long long capture_of(cudaStream_t s) {
+    if (s == nullptr || s == cudaStreamLegacy) return 0;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
     if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
@@ -248,15 +251,15 @@ unsigned long long capture_of(cudaStream_t s) {
 // The work just given to the stream leaves the forest flat, or not known to be.
 void set_flat(cc_ctx* c, bool flat) {
     const unsigned long long id = capture_of(c->stream);
-    if (id == 0) {
-        c->flat = flat;
+    if (id == 0 || id == kUnknown) {
+        c->flat = flat && id == 0;
         return;
     }
     if (id != c->rec_id) {
         c->replayable |= c->rec_id != 0 && !c->rec_flat;
         c->rec_id = id;
     }
-    c->rec_flat = flat && id != kUnknown;
+    c->rec_flat = flat;
 }
 
 // Whether the forest is flat for certain when the work given next runs: for work

@@ -200,3 +200,22 @@ def test_a_refused_call_does_not_fail_the_next(cc):
         assert ex.value.status == cc.CC_ERR_CUDA
     f.compress()
     assert f.components() == N
+
+
+def test_another_streams_capture_is_not_this_forests(cc):
+    """Nothing was recorded, so once the forest is compressed the two-kernel
+    Bulk-Find for flat forests is back."""
+    e = edges()[0]
+    ids = torch.arange(N, dtype=torch.int32, device="cuda")
+    f = cc.Forest(N, stream=0)
+    f.submit([(0, cc.OP_UPDATE, e, None)])
+    f.sync()
+    with foreign_capture():
+        with pytest.raises(cc.CCError):
+            f.submit([(0, cc.OP_UPDATE, e, None)])
+    f.compress()
+    before = f.kernel_stats()["query"]
+    found = f.bulk_find(ids)
+    torch.cuda.synchronize()
+    assert f.kernel_stats()["query"] - before == 2
+    assert np.array_equal(found.cpu().numpy(), np.arange(N) // 2 * 2)
