@@ -99,8 +99,8 @@ __device__ __forceinline__ void gather_parents(const int* parent, unsigned m, co
 #pragma unroll
     for (int i = 0; i < E; i++) {
         const bool on = (m >> i) & 1u;
-        pu[i] = on ? parent[u[i]] : u[i];
-        pv[i] = on ? parent[v[i]] : v[i];
+        pu[i] = on ? load_after(parent + u[i]) : u[i];
+        pv[i] = on ? load_after(parent + v[i]) : v[i];
     }
 }
 
@@ -524,14 +524,14 @@ k_update_live(int* __restrict__ parent, const int4* __restrict__ live, const uns
               int sel, DevState* __restrict__ ds, int hook) {
     pdl_trigger();
     pdl_wait();
-    const int64_t m = count[sel];
+    const int64_t m = (unsigned)load_after(reinterpret_cast<const int*>(count) + sel);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 2;
     int made = 0;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 2;
          WARP ? __any_sync(0xffffffffu, i < m) : i < m; i += stride) {
         const int4 zero = make_int4(0, 0, 0, 0);
-        const int4 a = i < m ? live[i] : zero;
-        const int4 b = i + 1 < m ? live[i + 1] : a;
+        const int4 a = i < m ? load_after(live + i) : zero;
+        const int4 b = i + 1 < m ? load_after(live + i + 1) : a;
         const unsigned on = i + 1 < m ? 3u : i < m ? 1u : 0u;
         const int u[2] = {a.x, b.x}, v[2] = {a.y, b.y}, pu[2] = {a.z, b.z}, pv[2] = {a.w, b.w};
         made += join_edges<2, WARP>(parent, on, u, v, pu, pv, ds, hook);
@@ -812,13 +812,13 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, con
     if constexpr (MODE == 2) {
 #pragma unroll
         for (int i = 0; i < E; i++) {
-            p[i] = act[i] ? __ldg(parent + hi[i]) : 0;
-            if (!LAZY) q[i] = act[i] ? __ldg(parent + lo[i]) : 0;
+            p[i] = act[i] ? load_after(parent + hi[i]) : 0;
+            if (!LAZY) q[i] = act[i] ? load_after(parent + lo[i]) : 0;
         }
         if (LAZY) {
 #pragma unroll
             for (int i = 0; i < E; i++)  // p > lo: lo's root is another; p == lo: lo is the root
-                q[i] = act[i] && p[i] < lo[i] ? __ldg(parent + lo[i]) : lo[i];
+                q[i] = act[i] && p[i] < lo[i] ? load_after(parent + lo[i]) : lo[i];
         }
 #pragma unroll
         for (int i = 0; i < E; i++)
@@ -834,8 +834,8 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, con
         for (int i = 0; i < E; i++) {
             p[i] = q[i] = 0;
             if (!act[i]) continue;
-            p[i] = MODE == 1 ? parent[hi[i]] : __ldg(parent + hi[i]);
-            q[i] = MODE == 1 ? parent[lo[i]] : __ldg(parent + lo[i]);
+            p[i] = load_after(parent + hi[i]);
+            q[i] = load_after(parent + lo[i]);
         }
 #pragma unroll
         for (int i = 0; i < E; i++) {
@@ -863,7 +863,7 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, con
         for (int i = 0; i < E; i++) {
             p[i] = 0;
             if (!act[i]) continue;
-            p[i] = MODE == 1 ? parent[hi[i]] : __ldg(parent + hi[i]);
+            p[i] = load_after(parent + hi[i]);
             any = true;
         }
         if (!any) break;
@@ -896,9 +896,9 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, con
 // so the pair loads (16 B per lane) and the answer stores (E bytes per lane)
 // are coalesced across the warp. The E walks of a thread advance in lockstep,
 // so their loads overlap.
-//  MODE 0: read-only finds through the read-only data path.
+//  MODE 0: read-only finds.
 //  MODE 1: finds with path splitting: every node walked over is repointed at
-//          its grandparent (they write, so ordinary loads).
+//          its grandparent.
 //  MODE 2: flat forest (every tree of height <= 1): the parents decide.
 // LAZY: see query_chunk.
 // PERSIST: a persistent grid that loads the next chunk's pairs before working
@@ -1003,8 +1003,8 @@ k_query_warp(const int* __restrict__ parent, int n, const int* __restrict__ pair
                         } else {
                             xu[j] = u;
                             xv[j] = v;
-                            pu[j] = __ldg(parent + u);
-                            pv[j] = __ldg(parent + v);
+                            pu[j] = load_after(parent + u);
+                            pv[j] = load_after(parent + v);
                             eq[j] = pu[j] == pv[j];
                         }
                     }
@@ -1025,11 +1025,11 @@ k_query_warp(const int* __restrict__ parent, int n, const int* __restrict__ pair
                 }
                 if (!eq[j] && pu[j] < xu[j]) {
                     xu[j] = pu[j];
-                    pu[j] = __ldg(parent + xu[j]);
+                    pu[j] = load_after(parent + xu[j]);
                 }
                 if (!eq[j] && pv[j] < xv[j]) {
                     xv[j] = pv[j];
-                    pv[j] = __ldg(parent + xv[j]);
+                    pv[j] = load_after(parent + xv[j]);
                 }
                 if (eq[j] || (pu[j] >= xu[j] && pv[j] >= xv[j])) {
                     if (!eq[j] && (pu[j] > xu[j] || pv[j] > xv[j])) corrupt = true;
