@@ -289,8 +289,10 @@ static cudaError_t launch(BulkFindState& b, int* parent, int n, const int* S, in
         const int64_t cap = resident_grid<k_bulk_find>(kBfBlock);
         void* args[] = {&S, &k, &n, &parent, &b.mark, &epoch, &b.front[0], &b.front[1], &b.roots,
                         &b.count, &res, &out, &ds};
-        e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_bulk_find),
-                                        dim3((unsigned)std::min(cap, need)), dim3(kBfBlock), args, 0, s);
+        e = launch_fitting((unsigned)std::min(cap, need), [&](unsigned grid) {
+            return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_bulk_find), dim3(grid),
+                                               dim3(kBfBlock), args, 0, s);
+        });
         if (e != cudaSuccess) return e;
         b.launches += 1;
     }

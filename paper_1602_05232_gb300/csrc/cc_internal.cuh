@@ -131,6 +131,20 @@ static void launch_windowed(void (*kernel)(Params...), unsigned grid, int block,
     launch_windowed_smem(kernel, grid, block, 0, s, window, pdl, args...);
 }
 
+// launch(grid), a cooperative launch, with fewer CTAs where that many cannot be
+// resident together: resident_grid counts all SMs of the device, and a stream or
+// a process may have a part of them only.
+template <class F>
+static cudaError_t launch_fitting(unsigned grid, F&& launch) {
+    cudaError_t e = launch(grid);
+    while (e == cudaErrorCooperativeLaunchTooLarge && grid > 1) {
+        cudaGetLastError();
+        grid = (grid + 1) / 2;
+        e = launch(grid);
+    }
+    return e;
+}
+
 // Whether work given to s is recorded into a graph instead of run (or may be:
 // the query fails on the legacy stream during another stream's capture).
 static inline bool capturing(cudaStream_t s) {
