@@ -499,7 +499,8 @@ cc_status cc_bulk_find(cc_ctx* ctx, const int32_t* S, int64_t k, int32_t* res);
 
 /* For the last Bulk-Find: the number of traversed non-root vertices
  * (|R_u| without R_0), and the number of Phase I and Phase II levels.
- * Synchronises. */
+ * Synchronises; CC_ERR_CUDA on a stream that is capturing, whose capture goes
+ * on. */
 cc_status cc_bulk_find_stats(cc_ctx* ctx, int64_t* traversed, int32_t* levels_up,
                              int32_t* levels_down);
 

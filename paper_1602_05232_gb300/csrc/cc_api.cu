@@ -1326,6 +1326,8 @@ cc_status cc_bulk_find_stats(cc_ctx* c, int64_t* traversed, int32_t* levels_up, 
     cc::BulkFindCounters h = {};
     if (c->bf.count) {
         CC_DEVICE(c);
+        if (cc::capturing(c->stream))  // without a call that would end the capture
+            return fail(CC_ERR_CUDA, "cc_bulk_find_stats: the stream is capturing, and the counts are on the device");
         cudaError_t e = cudaMemcpyAsync(&h, c->bf.count, sizeof h, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cc_bulk_find_stats");

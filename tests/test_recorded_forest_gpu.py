@@ -219,3 +219,24 @@ def test_another_streams_capture_is_not_this_forests(cc):
     torch.cuda.synchronize()
     assert f.kernel_stats()["query"] - before == 2
     assert np.array_equal(found.cpu().numpy(), np.arange(N) // 2 * 2)
+
+
+def test_statistics_asked_for_during_a_capture(cc):
+    """They are on the device, where a capture cannot wait for them; it is not ended."""
+    st = torch.cuda.Stream()
+    e, q = edges(), all_pairs()
+    out = torch.zeros(q.shape[0], dtype=torch.uint8, device="cuda")
+    f = cc.Forest(N, stream=st)
+    torch.cuda.synchronize()
+    f.bulk_find(q.view(-1))
+    stats = f.bulk_find_stats()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        deepen(f, e)
+        with pytest.raises(cc.CCError) as ex:
+            f.bulk_find_stats()
+        assert ex.value.status == cc.CC_ERR_CUDA
+        f.bulk_query(q, out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert out.all() and f.bulk_find_stats() == stats
