@@ -343,6 +343,12 @@ cc_status split_update(cc_ctx* c, const int32_t* edges, int64_t k, bool first, b
         c->live_cap = k;
     }
     const int sel = (int)(c->live_seq & 1u);
+    if (c->rec_id != 0 || capture_of(c->stream) != 0) {
+        // The counters alternate from call to call, each call clearing the next one's;
+        // a replayed graph's calls come in another order than they were made in.
+        e = cudaMemsetAsync(c->live_count + sel, 0, sizeof(unsigned), c->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "update variant 4: clear the list counter");
+    }
     cc::Launch cfg = update_cfg(c, first);
     if (ordered && cfg.pdl == 2) cfg.pdl = 1;  // its edges were written by the kernel just before
     cfg.alt = alt;

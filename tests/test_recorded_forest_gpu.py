@@ -240,3 +240,38 @@ def test_statistics_asked_for_during_a_capture(cc):
     g.replay()
     torch.cuda.synchronize()
     assert out.all() and f.bulk_find_stats() == stats
+
+
+@pytest.mark.parametrize("updates", [1, 2, 3])
+def test_two_pass_update_replayed(cc, updates):
+    """The list counter a replay appends through starts at zero each time."""
+    import oracle
+    r = np.random.default_rng(updates)
+    st = torch.cuda.Stream()
+    n, k = 20_000, 5_000
+    e = [torch.empty((k, 2), dtype=torch.int32, device="cuda") for _ in range(updates)]
+    f = cc.Forest(n, stream=st, update_variant=4, compress_every=0)
+    ref = oracle.OracleUF(n)
+
+    def fill():
+        for x in e:
+            p = r.integers(0, n, size=(k, 2)).astype(np.int32)
+            ref.bulk_update(p)
+            x.copy_(torch.from_numpy(p))
+        torch.cuda.synchronize()
+
+    fill()
+    for x in e:
+        f.bulk_update(x)            # the list is made here
+    torch.cuda.synchronize()
+    g = record(st, lambda: [f.bulk_update(x) for x in e])
+    for eager in (False, False, True, False):
+        fill()
+        if eager:
+            for x in e:
+                f.bulk_update(x)
+        else:
+            g.replay()
+        torch.cuda.synchronize()
+    assert np.array_equal(f.labels().cpu().numpy(), ref.labels())
+    f.sync()
