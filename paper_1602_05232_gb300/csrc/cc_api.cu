@@ -182,9 +182,18 @@ struct cc_ctx {
 
     // Bulk-Find (CC_OPT_BULK_FIND, cc_bulk_find)
     cc::BulkFindState bf;
+
+    std::vector<void*> kept;  // outgrown scratch that recorded work may still use
 };
 
 namespace {
+
+// Scratch that has been replaced by larger. On a handle that has been captured a
+// graph may still use it, so it stays until the handle is destroyed.
+void outgrow(cc_ctx* c, void* p) {
+    if (p && c->rec_id != 0) c->kept.push_back(p);
+    else cudaFree(p);
+}
 
 cudaEvent_t take_event(cc_ctx* c) {
     if (!c->spare.empty()) {
@@ -338,7 +347,7 @@ cc_status split_update(cc_ctx* c, const int32_t* edges, int64_t k, bool first, b
             cudaGetLastError();
             return fail(CC_ERR_OOM, "update variant 4: list of %lld edges", (long long)k);
         }
-        cudaFree(c->live);
+        outgrow(c, c->live);
         c->live = live;
         c->live_cap = k;
     }
@@ -383,7 +392,7 @@ cc_status order_edges(cc_ctx* c, const int32_t** edges, int64_t k, const unsigne
                 cudaGetLastError();
                 return fail(CC_ERR_OOM, "edge order: copy of %lld edges", (long long)k);
             }
-            cudaFree(c->order_buf);
+            outgrow(c, c->order_buf);
             c->order_buf = q;
             c->order_cap = k;
         }
@@ -394,7 +403,7 @@ cc_status order_edges(cc_ctx* c, const int32_t** edges, int64_t k, const unsigne
                 cudaGetLastError();
                 return fail(CC_ERR_OOM, "edge order: bucket counters");
             }
-            cudaFree(c->order_hist);
+            outgrow(c, c->order_hist);
             c->order_hist = q;
             c->order_hist_cap = counters;
         }
@@ -666,6 +675,7 @@ cc_status cc_destroy(cc_ctx* c) {
         cudaFree(c->order_buf);
         cudaFree(c->order_hist);
         cudaFree(c->big);
+        for (void* p : c->kept) cudaFree(p);
         cc::bulk_find_free(c->bf);
         if (c->window.num_bytes > 0) persist_release(c->device);
         cudaFree(c->parent);

@@ -275,3 +275,36 @@ def test_two_pass_update_replayed(cc, updates):
         torch.cuda.synchronize()
     assert np.array_equal(f.labels().cpu().numpy(), ref.labels())
     f.sync()
+
+
+@pytest.mark.parametrize("opts", [{"update_variant": 4}, {"edge_order": 6}, {"update_variant": 4, "edge_order": 9}])
+def test_replay_after_a_larger_call_has_outgrown_the_scratch(cc, opts):
+    import oracle
+    r = np.random.default_rng(3)
+    st = torch.cuda.Stream()
+    n, k = 50_000, 6_000
+    small = torch.empty((k, 2), dtype=torch.int32, device="cuda")
+    large = torch.empty((5 * k, 2), dtype=torch.int32, device="cuda")
+    f = cc.Forest(n, stream=st, **opts)
+    ref = oracle.OracleUF(n)
+
+    def fill(x):
+        p = r.integers(0, n, size=x.shape).astype(np.int32)
+        ref.bulk_update(p)
+        x.copy_(torch.from_numpy(p))
+        torch.cuda.synchronize()
+
+    fill(small)
+    f.bulk_update(small)
+    torch.cuda.synchronize()
+    g = record(st, lambda: f.bulk_update(small))
+    if "edge_order" in opts:
+        f.set_option("edge_order", 9)       # more buckets: the counters are outgrown too
+    fill(large)
+    f.bulk_update(large)
+    for _ in range(2):
+        fill(small)
+        g.replay()
+        torch.cuda.synchronize()
+    assert np.array_equal(f.labels().cpu().numpy(), ref.labels())
+    f.sync()
