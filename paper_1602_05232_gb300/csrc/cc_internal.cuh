@@ -255,7 +255,7 @@ struct SegLaunch {
     int smem_cap;  // graphs of at most this many vertices run in shared memory (<= 65536)
     int max_ctas;  // cap on the persistent grid (0 = one wave of resident CTAs)
     int grid = 0;  // set by prepare_segmented, as is
-    int depth = 0; // the chunks of pairs in shared memory per CTA (2 to 4)
+    int depth = 0; // the chunks of pairs in shared memory per CTA (2 to 4; 0 for one pair per thread)
 };
 
 // Sets the kernel's shared-memory attribute, the ring's depth and the persistent grid size.
