@@ -767,20 +767,18 @@ __device__ __forceinline__ void store_answers(uint8_t* __restrict__ out, int64_t
 // a largest-component bitmap, a pair whose endpoints are both marked is
 // answered 1 from the bitmap alone: it reads no parent and walks nothing.
 //
-// A pair is walked from its larger node only. Ids fall along every path, so
-// a root that is larger than the other side's node cannot be that side's root:
-// the pair is answered 0 there, and the other side is not read any further
-// (not at all, where the larger endpoint is itself a root). Otherwise the
-// larger node is replaced by its parent; nodes that meet answer 1. Every node
-// is read at most once, and none that walking both sides up to a verified root
-// would not read too. The kernel is bound by those gathers (one line per clock
-// and SM from L2, 71 G/s from DRAM), so what is not read is what it gains:
-// reading both endpoints and walking both to their roots, a pass over the
-// R-MAT stream (n = 2^24, 128 x 2^20 pairs, no compression) took 4.25 ms and
-// now takes 3.89; the 8192 x 8192 grid (32 x 2^22 pairs) 8.48 and now 7.01.
-//  LAZY: the smaller endpoint's parent is read only once the larger one's has
-//        not decided the pair. Otherwise both are read at once, which is a
-//        dependent read less where the pairs are too few to hide it.
+// Ids fall along every path, so a root that is larger than the other side's node
+// cannot be that side's root: the pair is answered 0 there, and the other side is
+// not read any further. Otherwise the larger node is replaced by its parent; nodes
+// that meet answer 1. Every node is read at most once.
+//  LAZY: only the larger node is moved up, and the smaller endpoint's parent is read
+//        only once the larger one's has not decided the pair. On a large forest the
+//        kernel is bound by the gathers (one line per clock and SM from L2, 71 G/s from
+//        DRAM), so what is not read is what it gains: reading both endpoints and walking
+//        both to their roots, a pass over the R-MAT stream (n = 2^24, 128 x 2^20 pairs,
+//        no compression) took 4.25 ms and now takes 3.89; the 8192 x 8192 grid (32 x 2^22
+//        pairs) 8.48 and now 7.01. Otherwise both nodes are read in a round and both
+//        moved up, which takes fewer rounds one after the other.
 template <int E, int MODE, bool LAZY>
 __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, const int (&u)[E], const int (&v)[E],
                                             int64_t e0, int64_t k, uint8_t (&a)[E],
@@ -861,32 +859,39 @@ __device__ __forceinline__ bool query_chunk(int* __restrict__ parent, int n, con
         bool any = false;
 #pragma unroll
         for (int i = 0; i < E; i++) {
-            p[i] = 0;
+            p[i] = q[i] = 0;
             if (!act[i]) continue;
             p[i] = load_after(parent + hi[i]);
+            q[i] = lo[i];
+            if constexpr (!LAZY) q[i] = load_after(parent + lo[i]);
             any = true;
         }
         if (!any) break;
 #pragma unroll
         for (int i = 0; i < E; i++) {
             if (!act[i]) continue;
-            if (p[i] >= hi[i]) {  // a root above lo's id, or a broken invariant: not connected
-                if (p[i] > hi[i]) flag(ds, ST_CORRUPT);
+            if (p[i] >= hi[i] || q[i] > lo[i]) {  // a root above lo's id, or a broken invariant: not connected
+                if (p[i] > hi[i] || q[i] > lo[i]) flag(ds, ST_CORRUPT);
                 act[i] = false;
                 continue;
             }
+            int beside = blo[i];
             if (MODE == 1 && bhi[i] >= 0) lower(parent, bhi[i], p[i]);  // splitting: skip a level
-            if (p[i] == lo[i]) {
+            if constexpr (!LAZY) {
+                if (MODE == 1 && blo[i] >= 0 && q[i] < lo[i]) lower(parent, blo[i], q[i]);
+                if (q[i] < lo[i]) beside = lo[i];
+            }
+            if (p[i] == lo[i] || p[i] == q[i]) {
                 a[i] = 1;
                 act[i] = false;
                 continue;
             }
-            const bool swap = p[i] < lo[i];
+            const bool swap = p[i] < q[i];
             const int below = hi[i];
-            hi[i] = swap ? lo[i] : p[i];
-            lo[i] = swap ? p[i] : lo[i];
-            bhi[i] = swap ? blo[i] : below;
-            blo[i] = swap ? below : blo[i];
+            hi[i] = swap ? q[i] : p[i];
+            lo[i] = swap ? p[i] : q[i];
+            bhi[i] = swap ? beside : below;
+            blo[i] = swap ? below : beside;
         }
     }
     return bad;
@@ -1069,11 +1074,15 @@ static void query_inst(unsigned g, Launch cfg, cudaStream_t s, int* parent, int 
 #undef CC_Q
 }
 
-// From this many pairs the second parent of a pair is read only if the first
-// does not decide it (LAZY of query_chunk). Always
-// lazy, 50,001 pairs on 10^6 vertices cost 0.1 us more a query; never lazy, the
-// R-MAT pass takes 4.23 instead of 3.89 ms and the grid 8.08 instead of 7.01.
+// LAZY of query_chunk from this many pairs and vertices. Fewer pairs leave the
+// latency of a round unhidden (50,001 on 10^6 vertices: 0.1 us more a query). Smaller
+// forests stay near the SMs: 2^20 pairs on a forest that two updates left deep, lazy
+// and not, 10.1 and 7.9 us for n = 2^10, 11.9 and 10.4 for 2^16, 14.4 and 13.7 for 2^20. On
+// larger ones, passes of 6 to 24 minibatches of 2^17 to 2^21 edges and pairs without
+// compression take 1.00 to 1.08 times as long without it for n = 2^22 to 2^24 and
+// 1.00 to 1.17 for 2^26.
 constexpr int64_t kLazyPairs = 1 << 17;
+constexpr int kLazyVertices = 1 << 22;
 
 cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_t* out,
                          DevState* ds, int mode, Launch cfg, cudaStream_t s) {
@@ -1093,7 +1102,8 @@ cudaError_t launch_query(int* parent, int n, const int* pairs, int64_t k, uint8_
     const int vec = pair_vec(pairs);
     const int ovec = (reinterpret_cast<uintptr_t>(out) % cfg.ept) == 0;
     const unsigned g = blocks_for(k, (int64_t)cfg.ept * cfg.block);
-#define CC_QM(M) if (k >= kLazyPairs) query_inst<M, true>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds); \
+    const bool lazy = k >= kLazyPairs && n >= kLazyVertices;
+#define CC_QM(M) if (lazy) query_inst<M, true>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds); \
                  else query_inst<M, false>(g, cfg, s, parent, n, pairs, k, vec, out, ovec, ds)
     switch (mode) {
         case 2: CC_QM(2); break;
