@@ -770,7 +770,7 @@ __device__ __forceinline__ void store_answers(uint8_t* __restrict__ out, int64_t
 // Ids fall along every path, so a root that is larger than the other side's node
 // cannot be that side's root: the pair is answered 0 there, and the other side is
 // not read any further. Otherwise the larger node is replaced by its parent; nodes
-// that meet answer 1. Every node is read at most once.
+// that meet answer 1.
 //  LAZY: only the larger node is moved up, and the smaller endpoint's parent is read
 //        only once the larger one's has not decided the pair. On a large forest the
 //        kernel is bound by the gathers (one line per clock and SM from L2, 71 G/s from
@@ -1077,7 +1077,7 @@ static void query_inst(unsigned g, Launch cfg, cudaStream_t s, int* parent, int 
 // LAZY of query_chunk from this many pairs and vertices. Fewer pairs leave the
 // latency of a round unhidden (50,001 on 10^6 vertices: 0.1 us more a query). Smaller
 // forests stay near the SMs: 2^20 pairs on a forest that two updates left deep, lazy
-// and not, 10.1 and 7.9 us for n = 2^10, 11.9 and 10.4 for 2^16, 14.4 and 13.7 for 2^20. On
+// and not, 9.5 and 7.9 us for n = 2^10, 12.0 and 10.5 for 2^16, 14.4 and 13.7 for 2^20. On
 // larger ones, passes of 6 to 24 minibatches of 2^17 to 2^21 edges and pairs without
 // compression take 1.00 to 1.08 times as long without it for n = 2^22 to 2^24 and
 // 1.00 to 1.17 for 2^26.
