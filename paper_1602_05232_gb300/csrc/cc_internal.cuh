@@ -35,6 +35,7 @@ struct DevState {
 enum : int {
     HOOK_MIN = 1,    // with atomicMin and a repair instead of a compare-and-swap
     HOOK_CLIMB = 2,  // under the other side's root, not just its node
+    HOOK_AGAIN = 4,  // a root among the first parents is read again before it is linked
 };
 
 struct Launch {

@@ -133,6 +133,13 @@ __device__ __forceinline__ void gather_parents(const int* parent, unsigned m, co
 // splitting store that races with the move and undoes it is harmless for the
 // same reason). Only a write at a root counts as a link. Each round strictly
 // lowers the larger node of every edge, so the loop ends.
+//
+// A first parent that was a root is tried without another read. With HOOK_AGAIN it
+// is read again first: where a minibatch has more edges than the graph vertices, most
+// of its edges are joined by others while they wait, and a try for each queues on the
+// few words that are left (2^18 edges on 4096 vertices with atomicMin, four
+// minibatches: 60 us with both roots verified first, 101 without a second read, 48
+// with it; 2^20 on 64 with compare-and-swap 354, 767 and 214).
 // One link attempt per distinct hi among the lanes of a whole warp that try
 // one: the first of them tries to put hi under its own lo. Returns hi if this
 // lane linked it, else hi's parent as this leaves it (p for a lane without a try).
@@ -153,8 +160,9 @@ template <int E, bool WARP>
 __device__ __forceinline__ int join_edges(int* parent, unsigned m, const int (&u)[E], const int (&v)[E],
                                           const int (&pu)[E], const int (&pv)[E], DevState* ds, int hook) {
     const bool minhook = hook & HOOK_MIN, climb = hook & HOOK_CLIMB;
+    const int root = hook & HOOK_AGAIN ? -2 : -1;
     int hi[E], lo[E];    // the two nodes of each edge; equal once it is done
-    int bhi[E], blo[E];  // the node below each on its path, or -1: it was a root when it was read
+    int bhi[E], blo[E];  // the node below each on its path, or -1: it was a root when it was read (-2: and is read again)
     bool any = false;
 #pragma unroll
     for (int i = 0; i < E; i++) {
@@ -162,8 +170,8 @@ __device__ __forceinline__ int join_edges(int* parent, unsigned m, const int (&u
         const int x = swap ? v[i] : u[i], y = swap ? u[i] : v[i];
         lo[i] = swap ? pu[i] : pv[i];
         hi[i] = !((m >> i) & 1u) ? lo[i] : swap ? pv[i] : pu[i];
-        bhi[i] = hi[i] == x ? -1 : x;
-        blo[i] = lo[i] == y ? -1 : y;
+        bhi[i] = hi[i] == x ? root : x;
+        blo[i] = lo[i] == y ? root : y;
         any |= hi[i] != lo[i];
     }
     int made = 0;
@@ -172,19 +180,19 @@ __device__ __forceinline__ int join_edges(int* parent, unsigned m, const int (&u
 #pragma unroll
         for (int i = 0; i < E; i++) {
             p[i] = hi[i];
-            if (hi[i] != lo[i] && bhi[i] >= 0) p[i] = parent[hi[i]];
+            if (hi[i] != lo[i] && bhi[i] != -1) p[i] = parent[hi[i]];
         }
         if (climb) {
             int q[E];
 #pragma unroll
             for (int i = 0; i < E; i++) {
                 q[i] = lo[i];
-                if (hi[i] != lo[i] && blo[i] >= 0 && p[i] == hi[i]) q[i] = parent[lo[i]];
+                if (hi[i] != lo[i] && blo[i] != -1 && p[i] == hi[i]) q[i] = parent[lo[i]];
             }
 #pragma unroll
             for (int i = 0; i < E; i++) {
                 if (q[i] >= lo[i]) continue;
-                lower(parent, blo[i], q[i]);
+                if (blo[i] >= 0) lower(parent, blo[i], q[i]);
                 blo[i] = lo[i];
                 lo[i] = q[i];
                 bhi[i] = -1;  // hi has been read and is a root
@@ -462,6 +470,12 @@ static void update_tiles_inst(const int* edges, int64_t k, int vec, int* parent,
                          (int)(pdl == 2), hook, fb);
 }
 
+// HOOK_AGAIN from this many edges per vertex. Four minibatches of 2^16 to 2^20
+// uniform or skewed edges on 16 to 2^18 vertices take 1.00 of the time with it at
+// half an edge per vertex, 0.92 at one, 0.86 at two, 0.82 at four and less from there;
+// but sixteen of 2^16 uniform edges on 2^16 vertices 1.01 to 1.02.
+static bool dense(int64_t k, int n) { return k >= 2 * (int64_t)n; }
+
 // --- VARIANT 4: filter pass + live-edge pass ------------------------------
 //
 // Once the forest is shallow, almost every edge of a minibatch already has
@@ -553,6 +567,7 @@ static void update_filter_inst(const int* edges, int64_t k, int vec, const int* 
 cudaError_t launch_update_split(int* parent, int n, const int* edges, int64_t k, DevState* ds, Launch cfg,
                                 int4* live, unsigned* count, int sel, cudaStream_t s) {
     if (k <= 0) return cudaSuccess;
+    if (dense(k, n)) cfg.hook |= HOOK_AGAIN;
     const int vec = pair_vec(edges);
     switch (cfg.ept) {
         case 1: update_filter_inst<1>(edges, k, vec, parent, n, live, count, sel, ds, cfg.block, cfg.window, cfg.pdl, BigArgs{cfg.big, cfg.alt}, s); break;
@@ -714,6 +729,7 @@ cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevSt
                           Launch cfg, cudaStream_t s) {
     if (k <= 0) return cudaSuccess;
     const int vec = pair_vec(edges);
+    if (dense(k, n)) cfg.hook |= HOOK_AGAIN;
     if (cfg.variant == 0 && k >= kTileEdges) {
         cfg.variant = 5;
         cfg.block = 128;
