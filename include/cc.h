@@ -80,12 +80,13 @@ typedef enum {
                                     later operations */
     CC_OPT_PROFILE = 5,          /* 1: time every kernel with CUDA events on the handle's stream */
     CC_OPT_UPDATE_VARIANT = 6,   /* Bulk-Update kernel: 0 = 1 for minibatches below 2^18 edges, 5 in
-                                    CTAs of 128 threads from there, and for up to 4096 edges on up
-                                    to 8192 vertices (without CC_OPT_EDGE_ORDER and
-                                    CC_OPT_BIG_FILTER) one CTA in shared memory, which also leaves
-                                    the forest compressed, whatever CC_OPT_COMPRESS_EVERY says; 1 = one chunk of edges per
-                                    thread; 2 = 1 on a persistent grid that prefetches the next edges, 3 = 2 that also has the next chunk's first
-                                    parent reads in flight during this chunk's walks, 4 = two
+                                    CTAs of 128 threads from there, and for up to 4096 edges (2048
+                                    where no compression is due) on up to 8192 vertices, without
+                                    CC_OPT_EDGE_ORDER and CC_OPT_BIG_FILTER, one CTA in shared
+                                    memory, which also leaves the forest compressed, whatever
+                                    CC_OPT_COMPRESS_EVERY says; 1 = one chunk of edges per thread;
+                                    2 = 1 on a persistent grid that prefetches the next edges, 3 =
+                                    2 that also has the next chunk's first parent reads in flight during this chunk's walks, 4 = two
                                     kernels: a filter pass that reads every edge's first parents
                                     and lists the edges whose parents differ (16 B each; the list,
                                     room for the largest minibatch so far, is allocated on first

@@ -740,7 +740,7 @@ cc_status cc_bulk_update(cc_ctx* c, const int32_t* edges, int64_t k) {
     const int32_t* given = edges;
     const bool fused = c->opt[CC_OPT_UPDATE_SCHEDULE] != 1;
     if (fused && c->opt[CC_OPT_UPDATE_VARIANT] == 0 && c->opt[CC_OPT_EDGE_ORDER] == 0 &&
-        c->opt[CC_OPT_BIG_FILTER] == 0 && cc::small_update(c->n, k)) {
+        c->opt[CC_OPT_BIG_FILTER] == 0 && cc::small_update(c->n, k, compress)) {
         s = run(c, CC_K_UPDATE, "bulk_update (small)", [&] {
             return cc::launch_update_small(c->parent, (int)c->n, edges, k, c->ds, (int)c->opt[CC_OPT_PDL], c->stream);
         });

@@ -178,9 +178,12 @@ cudaError_t launch_update(int* parent, int n, const int* edges, int64_t k, DevSt
 // at its root. Against the general update and its compression pass, whole steps
 // with a query each, the host enqueueing: 8.1-8.9 -> 6.0-6.9 us for up to 4096
 // edges on up to 4096 vertices and 1024 on 8192, 8.5 -> 8.1 for 4096 on 8192,
-// but 8.5 -> 10.3 for 8192 on 8192 and 8.7 -> 10.9 for 8192 on 4096.
+// but 8.5 -> 10.3 for 8192 on 8192 and 8.7 -> 10.9 for 8192 on 4096. Without a
+// compression due it saves no launch, and takes half as many edges: sixteen updates in
+// a row, nothing asked, on 16 to 8192 vertices 0.95 of the general ones' time with 2048
+// edges each, 1.15 with 3000 and 1.19 with 4096.
 constexpr int64_t kSmallVertices = 8192, kSmallEdges = 4096;
-bool small_update(int64_t n, int64_t k);
+bool small_update(int64_t n, int64_t k, bool compress);
 cudaError_t launch_update_small(int* parent, int n, const int* edges, int64_t k, DevState* ds, int pdl,
                                 cudaStream_t s);
 

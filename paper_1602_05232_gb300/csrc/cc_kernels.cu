@@ -705,7 +705,9 @@ k_update_small(int* __restrict__ parent, int n, const int* __restrict__ edges, i
     }
 }
 
-bool small_update(int64_t n, int64_t k) { return n <= kSmallVertices && k <= kSmallEdges; }
+bool small_update(int64_t n, int64_t k, bool compress) {
+    return n <= kSmallVertices && k <= (compress ? kSmallEdges : kSmallEdges / 2);
+}
 
 cudaError_t launch_update_small(int* parent, int n, const int* edges, int64_t k, DevState* ds, int pdl,
                                 cudaStream_t s) {
