@@ -125,9 +125,10 @@ typedef enum {
                                     conflict-free). Settable only while the forest has no edges;
                                     not for segmented handles. */
     CC_OPT_BULK_FIND = 15,       /* 1: Bulk-Query, and the relabel step of CC_OPT_UPDATE_SCHEDULE = 1,
-                                    find all their roots with ONE Bulk-Find (Algorithm 4), whose
-                                    path compression is shared by the whole minibatch (Theorem 3).
-                                    Default 0 */
+                                    find all their roots with ONE Bulk-Find (Algorithm 4), which
+                                    leaves the forest that its shared path compression leaves.
+                                    Each endpoint's path is walked for itself (not once for all
+                                    that share it, as Theorem 3 counts). Default 0 */
     CC_OPT_QUERY_VARIANT = 16,   /* Bulk-Query kernel: 0 = one chunk of pairs per thread (default),
                                     1 = a persistent grid that loads the next chunk's pairs while
                                     working on the current one, 2 = warp-cooperative: a warp takes
@@ -487,10 +488,12 @@ cc_status cc_copy_nonloop(cc_ctx* ctx, int32_t* out, int64_t cap, int64_t* count
 
 /* Bulk-Find (Algorithm 4; Section 4): res[i] = the root of S[i] for k
  * vertices `S` (device, k int32; an id outside [0, n) gives -1 and is
- * reported by cc_sync), with path compression shared by all of them:
- * afterwards every vertex on a path from some S[i] to its root points at that
- * root, and no other parent changes. Phase I walks up from all of S at once,
- * merging flows that meet; Phase II points every vertex met at its root.
+ * reported by cc_sync), with path compression for all of them: afterwards every
+ * vertex on a path from some S[i] to its root points at that root, and no other
+ * parent changes. Phase I walks up from all of S at once, merging flows that
+ * meet, and counts them; the roots come from a walk for each S[i], and Phase II
+ * points every vertex on it at its root. The work is the sum of the path
+ * lengths.
  * `res`: device, k int32 (it may be `S` itself). One cooperative kernel, or two
  * kernels when the forest is known to be flat (right after a full compression,
  * with no update since). Asynchronous, but for the scratch (12 bytes per vertex

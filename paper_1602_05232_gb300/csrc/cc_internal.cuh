@@ -62,11 +62,13 @@ struct Launch {
 // edges are dropped before their parent reads, and ordering them no longer
 // pays: launch_order_edges given the same `big` then does nothing, and an
 // update kernel given the ordered copy reads the caller's edges, `alt`,
-// instead. Both decide from big_root, which they may read before their own
-// wait for the kernel before them. Only the pick kernel and the reset write it,
-// and neither these nor the full compression pass that always follows the pick
-// (and waits for it) has a trigger: whatever is launched after them starts when
-// their CTAs have exited, and reads the final value.
+// instead. Both decide from big_root, which only the pick kernel and the reset
+// write. An update on an ordered copy always reads it after its wait (its pdl is
+// at most 1: the copy was written by the kernel just before). The count kernel of
+// the order may read it before its own; what it sees, past L1, is final all the
+// same, because neither the reset nor the full compression pass that always
+// follows the pick, and has waited for it, has a trigger: whatever is launched
+// after them starts when their CTAs have exited.
 struct BigArgs {
     const unsigned* big = nullptr;
     const int* alt = nullptr;

@@ -40,7 +40,7 @@ PLAIN_SPACE = {
     "block": [128, 256, 512, 1024],
     "compress_every": [0, 1, 2, 3, 4, 6, 8, 16],
     "compress_scope": [0, 1],
-    "query_halving": [0, 1, 2],
+    "query_halving": [0, 1],        # 2 is the same kernel as 1
     "l2_persist": [0, 1],
     "query_variant": [0, 1, 2],
     "pdl": [0, 1, 2],
